@@ -389,7 +389,7 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
 // region of at least the header (which holds the status word).
 struct OzPlan {
     int mt = 0, nt = 0, kt = 0, ks_a = 1, ks_b = 1;
-    size_t off_ea = 0, off_eb = 0, off_sa = 0, off_sb = 0, data_bytes = 0;
+    size_t off_exp = 0, off_a = 0, off_b = 0, data_bytes = 0;
 };
 
 OzPlan oz_plan(int64_t m, int64_t n, int64_t k, int slices)
@@ -397,19 +397,19 @@ OzPlan oz_plan(int64_t m, int64_t n, int64_t k, int slices)
     OzPlan o;
     o.mt = static_cast<int>((m + 127) / 128);
     o.nt = static_cast<int>((n + 127) / 128);
-    o.kt = static_cast<int>((k + 63) / 64);
-    // enough exponent-reduction blocks to cover the GPU (about 600), at most 64 k-ranges
+    o.kt = static_cast<int>((k + 31) / 32);
+    // enough exponent-reduction blocks to cover the GPU (about 600 an operand), at most 64
+    // k-ranges
     o.ks_a = std::max(1, std::min({64, o.kt, (600 + o.mt - 1) / std::max(1, o.mt)}));
     o.ks_b = std::max(1, std::min({64, o.kt, (600 + o.nt - 1) / std::max(1, o.nt)}));
+    const size_t plane = 128 * 32 * 2;
     size_t d = 0;
-    o.off_ea = d;
-    d += round_up((size_t)o.ks_a * o.mt * 128 * sizeof(int), kAlign);
-    o.off_eb = d;
-    d += round_up((size_t)o.ks_b * o.nt * 128 * sizeof(int), kAlign);
-    o.off_sa = d;
-    d += (size_t)slices * o.mt * o.kt * 16384;
-    o.off_sb = d;
-    d += (size_t)slices * o.nt * o.kt * 16384;
+    o.off_exp = d;
+    d += round_up((size_t)(o.mt + o.nt) * 128 * sizeof(int), kAlign);
+    o.off_a = d;
+    d += (size_t)slices * o.mt * o.kt * plane;
+    o.off_b = d;
+    d += (size_t)slices * o.nt * o.kt * plane;
     o.data_bytes = d;
     return o;
 }
@@ -1061,16 +1061,15 @@ int gfip_dgemm_ozaki(gfip_handle_t handle, char transa, char transb, int64_t m, 
     p.kt = o.kt;
     p.ks_a = o.ks_a;
     p.ks_b = o.ks_b;
-    p.ea = reinterpret_cast<int *>(data + o.off_ea);
-    p.eb = reinterpret_cast<int *>(data + o.off_eb);
-    p.sa = reinterpret_cast<uint16_t *>(data + o.off_sa);
-    p.sb = reinterpret_cast<uint16_t *>(data + o.off_sb);
+    p.exp = reinterpret_cast<int *>(data + o.off_exp);
+    p.pa = data + o.off_a;
+    p.pb = data + o.off_b;
     p.status = reinterpret_cast<unsigned int *>(h->ws);
     p.wait_ns = h->oz_wait_ns;
     p.inject_timeout = h->oz_inject;
-    if (gfip::launch_ozaki(p, h->stream) != cudaSuccess) return GFIP_ERR_CUDA;
-    h->last_launches = 5;
-    h->last_grid = o.mt * o.nt;
+    if (gfip::launch_ozaki(p, h->sms, h->stream) != cudaSuccess) return GFIP_ERR_CUDA;
+    h->last_launches = 3;
+    h->last_grid = static_cast<int>(std::min<int64_t>((int64_t)o.mt * o.nt, h->sms));
     return GFIP_OK;
 }
 

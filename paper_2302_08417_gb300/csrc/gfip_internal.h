@@ -118,6 +118,8 @@ template <typename T> struct GemmParams {
     unsigned int *done_count;        // CTAs of the current launch that have finished
     unsigned long long *pack_count;  // shared packing: epoch-tagged count of packed tiles
     unsigned long long *tile_next;   // epoch-tagged count of data-parallel tiles taken
+    unsigned int *gate;              // nullable (FP32): the launch does nothing while the word is
+                                     // zero, and clears it when it has run
 };
 
 // Parameters of the pack kernel of the pack-then-compute variant.
@@ -132,6 +134,47 @@ template <typename T> struct PackParams {
     T *pack_b;
 };
 
+// One launch of the tensor-core tile core (gfip_tc.cuh): both operands split into `planes`
+// BF16 planes, plane tiles of 128 rows x 32 k (8 KB, swizzled as the MMA reads them), laid out
+// [128-row block][k block][plane].
+struct TcParams {
+    const uint8_t *pa;   // planes of op(A), rows of C
+    const uint8_t *pb;   // planes of op(B), columns of C
+    void *C;             // double (digits) or float
+    int64_t ldc;
+    int m, n;
+    double alpha, beta;
+    int planes;
+    int mt, nt, kt;      // 128-row blocks of m and n, 32-wide k blocks
+    int tiles;           // tiles of C computed
+    int tri;             // TRI_*: the triangle of C computed (SYRK)
+    int tmask_a, tmask_b;  // triangular operand (TRMM): which k a tile needs, see TriMask
+    int splits;          // k-ranges per tile (FP32), added by the last to finish
+    int units;           // tiles * splits
+    const int *ea, *eb;  // digits: row exponents of op(A), column exponents of op(B)
+    float *partial;      // [tiles][splits] partial tiles of 128 x 128 (splits > 1)
+    unsigned int *counter;  // [tiles][8] arrivals, zero at launch (splits > 1)
+    const unsigned int *gate;  // nullable; the launch does nothing when the word is set
+    unsigned int *status;
+    unsigned long long wait_ns;  // budget of every mbarrier wait (nanoseconds)
+    int inject_timeout;  // test hook: CTA 0 withholds its first operand copy
+};
+
+// Large FP32 GEMMs on the tensor cores (gfip_f32_tc.cu): one operand of the split pass.
+struct F32SplitArgs {
+    const float *X;
+    int64_t ld;
+    int rows;         // rows of op(A) or columns of op(B)
+    int contig_rows;  // 1: element (r, p) at X[r + p*ld], 0: X[p + r*ld]
+    int row_blocks;   // 0: nothing to split (SYRK: B's planes are A's)
+    int mask;         // triangular operand (TRMM), 0 = dense; see TriMask
+    uint8_t *planes;
+};
+// Splits both operands and launches the tile core; an element outside the range of the split
+// sets *gate (which also makes the tile core do nothing).
+cudaError_t launch_f32_tc(const TcParams &p, const F32SplitArgs &a, const F32SplitArgs &b, int k,
+                          unsigned int *gate, int sms, cudaStream_t s);
+
 // FP64 GEMM emulated with BF16 digit products on the tensor cores (gfip_ozaki.cu).
 struct OzakiParams {
     const double *A;
@@ -143,18 +186,16 @@ struct OzakiParams {
     int a_contig_rows;   // 1: row i of op(A) runs along memory (transa 'N')
     int b_contig_rows;   // 1: column j of op(B) = row j of its K-major form runs along memory ('T')
     int slices;          // digits per element (S)
-    int mt, nt, kt;      // 128-row blocks of m and n, 64-wide k blocks
+    int mt, nt, kt;      // 128-row blocks of m and n, 32-wide k blocks
     int ks_a, ks_b;      // k-ranges the exponent reductions are split into
-    int *ea;             // [ks_a][mt * 128] partial row exponents of op(A)
-    int *eb;             // [ks_b][nt * 128] partial column exponents of op(B)
-    uint16_t *sa;        // [S][mt][kt] digit tiles of op(A), 16 KB each
-    uint16_t *sb;        // [S][nt][kt] digit tiles of op(B)
+    int *exp;            // [(mt + nt) * 128] row exponents of op(A), column exponents of op(B)
+    uint8_t *pa;         // digit planes of op(A)
+    uint8_t *pb;         // digit planes of op(B)
     unsigned int *status;
     unsigned long long wait_ns;  // budget of every mbarrier wait (nanoseconds)
     int inject_timeout;  // test hook: CTA 0 withholds its first operand copy
 };
-cudaError_t launch_ozaki(const OzakiParams &p, cudaStream_t s);
-size_t ozaki_smem_bytes();
+cudaError_t launch_ozaki(const OzakiParams &p, int sms, cudaStream_t s);
 
 // Triangular solve (gfip_trsm.cu): one launch solves a panel of at most TRSM_PANEL unknowns
 // (op(A)'s diagonal block at (k0, k0), transposed for side 'R') for every right-hand side;
