@@ -19,6 +19,14 @@
  * SUP path) and a pack-then-compute pair of launches (the conventional path).  All three
  * produce bit-identical results for the same arguments on the same GPU.
  *
+ * FP32 products of at least 2^21 multiply-adds, 64 rows, columns and terms run on the tensor
+ * cores in every routine (GEMM in all three variants, SYRK, TRMM, TRSM updates): packing splits
+ * each operand exactly into three BF16 planes, whose products are summed in FP32; the error
+ * against the exact product is no larger than that of FP32 multiply-adds.  Operands with an
+ * infinity, a NaN or a nonzero magnitude outside [2^-100, 2^55) are multiplied by the FP32
+ * kernel above, decided on the device.  A workspace too small for the planes (see
+ * gfip_workspace_size) but large enough for that kernel runs there too.
+ *
  * Pointers: A, B and C are DEVICE pointers owned by the caller; A and B are only read;
  * only the m x n logical region of C is written (rows m..ldc-1 are never touched).  Calls
  * are asynchronous on the handle's stream.
@@ -73,7 +81,7 @@ typedef struct gfip_handle_s *gfip_handle_t;
 #define GFIP_STATUS_BAD_SEGMENT 0x1u   /* a split tile saw more partial sums than planned */
 #define GFIP_STATUS_MMA_TIMEOUT 0x2u   /* gfip_dgemm_ozaki: a pipeline wait gave up (result invalid) */
 #define GFIP_STATUS_BAD_PROBLEM 0x4u   /* grouped GEMM: a problem had invalid arguments (skipped)  */
-#define GFIP_STATUS_WAIT_TIMEOUT 0x8u  /* FP32 GEMM: a pipeline wait of the warp-specialised tile
+#define GFIP_STATUS_WAIT_TIMEOUT 0x8u  /* FP32 GEMM: a pipeline wait of a warp-specialised tile
                                           core gave up (result invalid)                          */
 
 /* Pack policies for gfip_set_pack_policy(). */

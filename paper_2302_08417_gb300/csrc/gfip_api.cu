@@ -25,12 +25,20 @@ constexpr size_t kLaunchCountOffset = 64;   // header word: GEMM launches so far
 constexpr size_t kDoneCountOffset = 128;    // header word: finished CTAs of the running launch
 constexpr size_t kPackCountOffset = 192;    // header word: tiles packed by shared packing
 constexpr size_t kTileNextOffset = 32;      // header word: data-parallel tiles taken
+constexpr size_t kGateOffset = 48;          // header word: FP32 operands outside the split's range
 constexpr size_t kCtrlGranule = 64 * 1024;  // control region grows in these steps
 constexpr int kMinSplitRun = 8;              // shortest k run per CTA in a split wave
 // Split tiles of an FP32 launch with fewer tiles than CTAs: each CTA takes at least this many
 // k-blocks, so a 128 x 128 tile is summed from a few partial tiles, not from one per k-block.
 constexpr int kMinSplitRunF32 = 4;
 constexpr unsigned long long kOzakiWaitNs = 2000000000ull;  // 2 s per pipeline wait
+// FP32 products of at least this many multiply-adds, and this many rows, columns and terms, run
+// on the tensor cores (gfip_f32_tc.cu).  Its three launches take 16 us at 128^3, where the FFMA
+// core, splitting one tile's k over CTAs, takes 23; at 512^3 24 against 60, at 2048^3 109
+// against 369, at 64 x 8192 x 8192 223 against 405 (us, device time, one GB300).
+constexpr int64_t kTcMinWork = 1 << 21;
+constexpr int64_t kTcMinDim = 64;
+constexpr int64_t kTcMaxK = 1 << 17;   // sums of k products stay in FP32's range (gfip_f32_tc.cu)
 
 struct Handle {
     uint32_t magic = kMagic;
@@ -237,6 +245,58 @@ template <typename T> size_t total_bytes(Handle *h, const Plan<T> &pl)
     return ctrl + pl.data_bytes;
 }
 
+// A large FP32 product on the tensor cores (gfip_f32_tc.cu): the split pass, then the tile
+// core over the plane tiles, k split over `splits` units per tile.
+struct TcPlan {
+    bool use = false;
+    int mt = 0, nt = 0, kt = 0, tiles = 0, splits = 1;
+    size_t off_a = 0, off_b = 0, off_partial = 0, off_counter = 0, data_bytes = 0;
+};
+
+template <typename T>
+TcPlan tc_plan(const Handle *h, int64_t m, int64_t n, int64_t k, int tri)
+{
+    TcPlan t;
+    if (sizeof(T) != 4 || k > kTcMaxK || m * n * k < kTcMinWork || std::min({m, n, k}) < kTcMinDim)
+        return t;
+    t.use = true;
+    t.mt = static_cast<int>((m + 127) / 128);
+    t.nt = static_cast<int>((n + 127) / 128);
+    t.kt = static_cast<int>((k + 31) / 32);
+    t.tiles = tri ? t.mt * (t.mt + 1) / 2 : t.mt * t.nt;
+    // The units of one tile run on different SMs.  Fewest k blocks in a row on the busiest SM,
+    // each unit costing about 6 more (pipeline fill, epilogue), a split tile 2 per part added.
+    int64_t best = std::numeric_limits<int64_t>::max();
+    for (int s = 1; s <= 16 && s * 4 <= std::max(4, t.kt); ++s) {
+        const int64_t rounds = ((int64_t)t.tiles * s + h->sms - 1) / h->sms;
+        const int64_t cost = rounds * ((t.kt + s - 1) / s + 6) + (s > 1 ? 4 + 2 * s : 0);
+        if (cost < best) {
+            best = cost;
+            t.splits = s;
+        }
+    }
+    const size_t plane = 128 * 32 * 2;
+    size_t d = 0;
+    t.off_a = d;
+    d += (size_t)3 * t.mt * t.kt * plane;
+    t.off_b = tri ? t.off_a : d;
+    if (!tri) d += (size_t)3 * t.nt * t.kt * plane;
+    t.off_partial = d;
+    if (t.splits > 1) d += (size_t)t.tiles * t.splits * 128 * 128 * sizeof(float);
+    t.off_counter = d;
+    if (t.splits > 1) d += round_up((size_t)t.tiles * 8 * sizeof(unsigned int), kAlign);
+    t.data_bytes = d;
+    return t;
+}
+
+// Workspace a call needs: the plan's control words, and the data of whichever path runs (the
+// FFMA launch behind the tensor-core path reuses the same bytes).
+template <typename T> size_t call_bytes(Handle *h, const Plan<T> &pl, const TcPlan &t)
+{
+    const size_t ctrl = std::max(h->ctrl_bytes, round_up(pl.ctrl_needed, kCtrlGranule));
+    return ctrl + std::max(pl.data_bytes, t.data_bytes);
+}
+
 // Grows the handle's control region to `want` bytes.  The new part may hold data of earlier
 // calls, so it is cleared with a memset ordered on the handle's stream after them.  That
 // memset must not be recorded into a CUDA graph: a replay would clear the launch counter and
@@ -263,7 +323,8 @@ bool too_big(int64_t v)
 template <typename T>
 int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t m, int64_t n,
                 int64_t k, T alpha, const T *A, int64_t lda, const T *B, int64_t ldb, T beta,
-                T *C, int64_t ldc, int tmask_a = 0, int tmask_b = 0);
+                T *C, int64_t ldc, int tmask_a = 0, int tmask_b = 0,
+                size_t ws_limit = std::numeric_limits<size_t>::max());
 
 template <typename T>
 int gemm_entry(gfip_handle_t handle, Variant v, char transa, char transb, int64_t m, int64_t n,
@@ -293,16 +354,61 @@ int gemm_entry(gfip_handle_t handle, Variant v, char transa, char transb, int64_
                           beta, C, ldc);
 }
 
+// The split pass and the tensor-core tile core of one FP32 product described by p.
+cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<float> &p,
+                      unsigned char *data)
+{
+    gfip::TcParams q{};
+    q.pa = data + t.off_a;
+    q.pb = data + t.off_b;
+    q.C = p.C;
+    q.ldc = p.ldc;
+    q.m = p.m;
+    q.n = p.n;
+    q.alpha = p.alpha;
+    q.beta = p.beta;
+    q.planes = 3;
+    q.mt = t.mt;
+    q.nt = t.nt;
+    q.kt = t.kt;
+    q.tiles = t.tiles;
+    q.tri = p.tri;
+    q.tmask_a = p.tmask_a;
+    q.tmask_b = p.tmask_b;
+    q.splits = t.splits;
+    q.units = t.tiles * t.splits;
+    q.partial = reinterpret_cast<float *>(data + t.off_partial);
+    q.counter = reinterpret_cast<unsigned int *>(data + t.off_counter);
+    q.gate = p.gate;
+    q.status = p.status;
+    q.wait_ns = kOzakiWaitNs;
+    const gfip::F32SplitArgs a{p.A, p.lda, p.m, p.a_contig_m, t.mt, p.tmask_a, data + t.off_a};
+    gfip::F32SplitArgs b{p.B, p.ldb, p.n, p.b_contig_n, t.nt, p.tmask_b, data + t.off_b};
+    if (p.tri != gfip::TRI_NONE) b.row_blocks = 0;   // both roles read the planes of A
+    return gfip::launch_f32_tc(q, a, b, p.k, p.gate, h->sms, h->stream);
+}
+
 // Plans and launches one GEMM (or the triangle `tri` of one) whose arguments are checked
 // and whose quick returns are taken.
 template <typename T>
 int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t m, int64_t n,
                 int64_t k, T alpha, const T *A, int64_t lda, const T *B, int64_t ldb, T beta,
-                T *C, int64_t ldc, int tmask_a, int tmask_b)
+                T *C, int64_t ldc, int tmask_a, int tmask_b, size_t ws_limit)
 {
-    Plan<T> pl = make_plan<T>(h, v, (int)m, (int)n, (int)k, tri, tmask_a || tmask_b);
     if (h->ws == nullptr) return GFIP_ERR_WORKSPACE;
-    if (total_bytes(h, pl) > h->ws_bytes) return GFIP_ERR_WORKSPACE;
+    ws_limit = std::min(ws_limit, h->ws_bytes);
+    // A workspace too small for the split planes still serves the FFMA path.
+    TcPlan tc = tc_plan<T>(h, m, n, k, tri);
+    if (tc.use) {
+        // The FFMA launch behind it runs only for operands outside the split's range, so the
+        // separate pack pass of pack-then-compute (same bits) is left out.
+        const Variant w = v == Variant::PackThenCompute ? Variant::Direct : v;
+        const Plan<T> behind = make_plan<T>(h, w, (int)m, (int)n, (int)k, tri, tmask_a || tmask_b);
+        tc.use = call_bytes(h, behind, tc) <= ws_limit;
+        if (tc.use) v = w;
+    }
+    Plan<T> pl = make_plan<T>(h, v, (int)m, (int)n, (int)k, tri, tmask_a || tmask_b);
+    if (total_bytes(h, pl) > ws_limit) return GFIP_ERR_WORKSPACE;
 
     // Grow the control region if this plan needs more of it.
     if (const int rc = grow_ctrl(h, round_up(pl.ctrl_needed, kCtrlGranule)); rc != GFIP_OK)
@@ -359,6 +465,13 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
     p.tile_next = reinterpret_cast<unsigned long long *>(h->ws + kTileNextOffset);
 
     int launches = 0;
+    if constexpr (sizeof(T) == 4) {
+        if (tc.use) {
+            p.gate = reinterpret_cast<unsigned int *>(h->ws + kGateOffset);
+            if (launch_tc(h, tc, p, data) != cudaSuccess) return GFIP_ERR_CUDA;
+            launches += 2;
+        }
+    }
     if (v == Variant::PackThenCompute) {
         gfip::PackParams<T> pp{};
         pp.A = A;
@@ -458,7 +571,7 @@ size_t workspace_size_impl(Handle *h, char transa, char transb, int64_t m, int64
     if (too_big(m) || too_big(n) || too_big(k)) return 0;
     if (m == 0 || n == 0 || k == 0) return round_up(kHeader, kCtrlGranule);
     const Plan<T> pl = make_plan<T>(h, v, (int)m, (int)n, (int)k);
-    return total_bytes(h, pl);
+    return call_bytes(h, pl, tc_plan<T>(h, m, n, k, gfip::TRI_NONE));
 }
 
 // Reference-BLAS dsyrk argument check: 0, or minus the 1-based position of the first bad
@@ -522,7 +635,7 @@ size_t syrk_workspace_impl(Handle *h, char uplo, char trans, int64_t n, int64_t 
     if (n == 0 || k == 0) return round_up(kHeader, kCtrlGranule);
     const int tri = (uplo == 'L' || uplo == 'l') ? gfip::TRI_LOWER : gfip::TRI_UPPER;
     const Plan<T> pl = make_plan<T>(h, Variant::Fused, (int)n, (int)n, (int)k, tri);
-    return total_bytes(h, pl);
+    return call_bytes(h, pl, tc_plan<T>(h, n, n, k, tri));
 }
 
 // Reference-BLAS dtrmm argument check: 0, or minus the 1-based position of the first bad
@@ -563,7 +676,8 @@ size_t trmm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
     const bool left = side == 'L' || side == 'l';
     const Plan<T> pl =
         make_plan<T>(h, Variant::Fused, (int)m, (int)n, (int)(left ? m : n), gfip::TRI_NONE, true);
-    return round_up(total_bytes(h, pl), kAlign) + round_up((size_t)m * n * sizeof(T), kAlign);
+    const TcPlan tc = tc_plan<T>(h, m, n, left ? m : n, gfip::TRI_NONE);
+    return round_up(call_bytes(h, pl, tc), kAlign) + round_up((size_t)m * n * sizeof(T), kAlign);
 }
 
 // TRMM on the fused kernel: W := alpha op(A) B (or alpha B op(A)) with op(A) read through a
@@ -597,8 +711,11 @@ int trmm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     const int64_t kdim = left ? m : n;
     const Plan<T> pl =
         make_plan<T>(h, Variant::Fused, (int)m, (int)n, (int)kdim, gfip::TRI_NONE, true);
-    const size_t w_off = round_up(total_bytes(h, pl), kAlign);
     const size_t w_bytes = (size_t)m * n * sizeof(T);
+    // a workspace without room for the split planes of the tensor-core path runs without it
+    size_t w_off =
+        round_up(call_bytes(h, pl, tc_plan<T>(h, m, n, kdim, gfip::TRI_NONE)), kAlign);
+    if (w_off + w_bytes > h->ws_bytes) w_off = round_up(total_bytes(h, pl), kAlign);
     if (w_off + w_bytes > h->ws_bytes) return GFIP_ERR_WORKSPACE;
     T *W = reinterpret_cast<T *>(h->ws + w_off);
     const size_t row_bytes = (size_t)m * sizeof(T);
@@ -609,9 +726,9 @@ int trmm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     const int mask = trmm_mask(side, uplo, transa, diag);
     const char ta = is_notrans(transa) ? 'N' : 'T';
     const int rc = left ? launch_plan<T>(h, Variant::Fused, gfip::TRI_NONE, ta, 'N', m, n, m,
-                                         alpha, A, lda, B, ldb, beta, W, m, mask, 0)
+                                         alpha, A, lda, B, ldb, beta, W, m, mask, 0, w_off)
                         : launch_plan<T>(h, Variant::Fused, gfip::TRI_NONE, 'N', ta, m, n, n,
-                                         alpha, B, ldb, A, lda, beta, W, m, 0, mask);
+                                         alpha, B, ldb, A, lda, beta, W, m, 0, mask, w_off);
     if (rc != GFIP_OK) return rc;
     if (cudaMemcpy2DAsync(B, (size_t)ldb * sizeof(T), W, row_bytes, row_bytes, (size_t)n,
                           cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess)
@@ -619,8 +736,9 @@ int trmm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     return GFIP_OK;
 }
 
+// Workspace every panel update of a TRSM can run in (the FFMA or DFMA path's).
 template <typename T>
-size_t trsm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
+size_t trsm_workspace_min(Handle *h, char side, int64_t m, int64_t n)
 {
     // every update is at most all of B (m x n) against one panel of unknowns, and its plan's
     // workspace grows with each dimension
@@ -629,6 +747,30 @@ size_t trsm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
     const Plan<T> panel =
         make_plan<T>(h, Variant::Fused, (int)m, (int)n, std::min(gfip::TRSM_PANEL, na));
     return total_bytes(h, panel);
+}
+
+// ... and with room for the tensor-core path of the updates that take it.
+template <typename T>
+size_t trsm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
+{
+    const bool left = side == 'L' || side == 'l';
+    const int64_t na = left ? m : n;
+    size_t bytes = trsm_workspace_min<T>(h, side, m, n);
+    if (sizeof(T) == 4) {
+        auto update = [&](int64_t rest, int64_t width) {
+            const int64_t um = left ? rest : m, un = left ? n : rest;
+            const Plan<T> pl = make_plan<T>(h, Variant::Fused, (int)um, (int)un, (int)width);
+            bytes =
+                std::max(bytes, call_bytes(h, pl, tc_plan<T>(h, um, un, width, gfip::TRI_NONE)));
+        };
+        // forward, the unknowns after each whole panel; backward, those before each panel
+        for (int64_t p0 = 0; p0 < na; p0 += gfip::TRSM_PANEL) {
+            const int64_t width = std::min<int64_t>(gfip::TRSM_PANEL, na - p0);
+            if (p0 + width < na) update(na - p0 - width, width);
+            if (p0 > 0) update(p0, width);
+        }
+    }
+    return bytes;
 }
 
 // TRSM, blocked: B := alpha B, then over panels of op(A)'s diagonal in solve order (forward
@@ -655,7 +797,7 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
         // every check before the first launch
         if (A == nullptr) return GFIP_ERR_NULLPTR;
         if (h->ws == nullptr) return GFIP_ERR_WORKSPACE;
-        if (trsm_workspace_impl<T>(h, side, m, n) > h->ws_bytes) return GFIP_ERR_WORKSPACE;
+        if (trsm_workspace_min<T>(h, side, m, n) > h->ws_bytes) return GFIP_ERR_WORKSPACE;
     }
     if (alpha != T(1)) {   // B := alpha B (alpha == 0: zeros, B not read)
         if (gfip::launch_scale<T>(B, ldb, (int)m, (int)n, alpha, gfip::TRI_NONE, h->stream) !=

@@ -1088,6 +1088,9 @@ __global__ void __launch_bounds__(TileCfg<T>::THREADS, TileCfg<T>::MIN_BLOCKS)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     GemmSmem<T> &sm = *reinterpret_cast<GemmSmem<T> *>(smem_raw);
+    if constexpr (sizeof(T) == 4) {   // the tensor-core launch before this one did the work
+        if (p.gate != nullptr && *(volatile unsigned int *)p.gate == 0u) return;
+    }
     unsigned int epoch = 0u;
     if (threadIdx.x == 0) epoch = *(volatile unsigned int *)p.launch_count + 1u;
     Kernel<T, ACONTIG, BCONTIG, TileCfg<T>, TMASK>::run(p, sm, epoch);
@@ -1096,6 +1099,9 @@ __global__ void __launch_bounds__(TileCfg<T>::THREADS, TileCfg<T>::MIN_BLOCKS)
         if (atomicAdd(p.done_count, 1u) == gridDim.x - 1) {
             *(volatile unsigned int *)p.done_count = 0u;
             *(volatile unsigned int *)p.launch_count = epoch;
+            if constexpr (sizeof(T) == 4) {
+                if (p.gate != nullptr) *(volatile unsigned int *)p.gate = 0u;
+            }
             __threadfence();
         }
     }

@@ -757,6 +757,8 @@ __global__ void __launch_bounds__(THREADS, 1) ws_gemm_kernel(const GemmParams<fl
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int warp = threadIdx.x >> 5;
     const int wg = warp >> 2;
+    // the tensor-core launch before this one has computed the product
+    if (p.gate != nullptr && *(volatile unsigned int *)p.gate == 0u) return;
     if (threadIdx.x == 0) {
         for (int r = 0; r < VCTA; ++r)
             for (int s = 0; s < STAGES; ++s) {
@@ -790,6 +792,7 @@ __global__ void __launch_bounds__(THREADS, 1) ws_gemm_kernel(const GemmParams<fl
             const unsigned int epoch = *(volatile unsigned int *)p.launch_count + 1u;
             *(volatile unsigned int *)p.done_count = 0u;
             *(volatile unsigned int *)p.launch_count = epoch;
+            if (p.gate != nullptr) *(volatile unsigned int *)p.gate = 0u;
             __threadfence();
         }
     }
