@@ -19,12 +19,16 @@
  * SUP path) and a pack-then-compute pair of launches (the conventional path).  All three
  * produce bit-identical results for the same arguments on the same GPU.
  *
- * FP32 products of at least 2^21 multiply-adds, 64 rows, columns and terms run on the tensor
- * cores in every routine (GEMM in all three variants, SYRK, TRMM, TRSM updates): packing splits
+ * Small products, whose panels are not reused enough to pay for packing, run in one launch that
+ * reads both operands where they lie; in every routine and variant alike (FP64: up to 2^35
+ * multiply-adds unless C is large and k at most 64; FP32: where it is estimated fastest).
+ *
+ * Other FP32 products of at least 16 terms run on the tensor cores in every routine (GEMM in all
+ * three variants, SYRK, TRMM, TRSM updates): packing splits
  * each operand exactly into three BF16 planes, whose products are summed in FP32; the error
  * against the exact product is no larger than that of FP32 multiply-adds.  Operands with an
  * infinity, a NaN or a nonzero magnitude outside [2^-100, 2^55) are multiplied by the FP32
- * kernel above, decided on the device.  A workspace too small for the planes (see
+ * kernel described first, decided on the device.  A workspace too small for the planes (see
  * gfip_workspace_size) but large enough for that kernel runs there too.
  *
  * Pointers: A, B and C are DEVICE pointers owned by the caller; A and B are only read;

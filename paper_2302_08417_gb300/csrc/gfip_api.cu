@@ -32,12 +32,9 @@ constexpr int kMinSplitRun = 8;              // shortest k run per CTA in a spli
 // k-blocks, so a 128 x 128 tile is summed from a few partial tiles, not from one per k-block.
 constexpr int kMinSplitRunF32 = 4;
 constexpr unsigned long long kOzakiWaitNs = 2000000000ull;  // 2 s per pipeline wait
-// FP32 products of at least this many multiply-adds, and this many rows, columns and terms, run
-// on the tensor cores (gfip_f32_tc.cu).  Its three launches take 16 us at 128^3, where the FFMA
-// core, splitting one tile's k over CTAs, takes 23; at 512^3 24 against 60, at 2048^3 109
-// against 369, at 64 x 8192 x 8192 223 against 405 (us, device time, one GB300).
-constexpr int64_t kTcMinWork = 1 << 21;
-constexpr int64_t kTcMinDim = 64;
+// FP32 products of at least this many terms may run on the tensor cores (gfip_f32_tc.cu): with
+// fewer, the terms the split leaves out would show beside the rounding of the sum.
+constexpr int64_t kTcMinK = 16;
 constexpr int64_t kTcMaxK = 1 << 17;   // sums of k products stay in FP32's range (gfip_f32_tc.cu)
 
 struct Handle {
@@ -250,6 +247,7 @@ template <typename T> size_t total_bytes(Handle *h, const Plan<T> &pl)
 struct TcPlan {
     bool use = false;
     int mt = 0, nt = 0, kt = 0, tiles = 0, splits = 1;
+    int64_t cost = 0;   // k blocks in a row on the busiest SM, overheads counted as blocks
     size_t off_a = 0, off_b = 0, off_partial = 0, off_counter = 0, data_bytes = 0;
 };
 
@@ -257,8 +255,7 @@ template <typename T>
 TcPlan tc_plan(const Handle *h, int64_t m, int64_t n, int64_t k, int tri)
 {
     TcPlan t;
-    if (sizeof(T) != 4 || k > kTcMaxK || m * n * k < kTcMinWork || std::min({m, n, k}) < kTcMinDim)
-        return t;
+    if (sizeof(T) != 4 || k > kTcMaxK || k < kTcMinK) return t;
     t.use = true;
     t.mt = static_cast<int>((m + 127) / 128);
     t.nt = static_cast<int>((n + 127) / 128);
@@ -266,12 +263,12 @@ TcPlan tc_plan(const Handle *h, int64_t m, int64_t n, int64_t k, int tri)
     t.tiles = tri ? t.mt * (t.mt + 1) / 2 : t.mt * t.nt;
     // The units of one tile run on different SMs.  Fewest k blocks in a row on the busiest SM,
     // each unit costing about 6 more (pipeline fill, epilogue), a split tile 2 per part added.
-    int64_t best = std::numeric_limits<int64_t>::max();
+    t.cost = std::numeric_limits<int64_t>::max();
     for (int s = 1; s <= 16 && s * 4 <= std::max(4, t.kt); ++s) {
         const int64_t rounds = ((int64_t)t.tiles * s + h->sms - 1) / h->sms;
         const int64_t cost = rounds * ((t.kt + s - 1) / s + 6) + (s > 1 ? 4 + 2 * s : 0);
-        if (cost < best) {
-            best = cost;
+        if (cost < t.cost) {
+            t.cost = cost;
             t.splits = s;
         }
     }
@@ -287,6 +284,33 @@ TcPlan tc_plan(const Handle *h, int64_t m, int64_t n, int64_t k, int tri)
     if (t.splits > 1) d += round_up((size_t)t.tiles * 8 * sizeof(unsigned int), kAlign);
     t.data_bytes = d;
     return t;
+}
+
+// Whether a product runs on the small kernels (gfip_small.cu).
+//
+// FP64: everywhere but where the persistent core is as fast.  Above 2^35 multiply-adds both are
+// DFMA-bound within 0.1 % (4096^3: 109.9 and 110.0 ms) and the core draws a tenth of the L2
+// traffic; with few terms per element of a large C its 32 x 32 tiles cost less around the
+// arithmetic (8192 x 8192 x 64: 7.19 ms against 7.27; 1500 x 1500 x 64: 272 us against 251).
+//
+// FP32: where the estimated time, in ns, is below the tensor cores' (or the FFMA core's, where
+// those cannot be used).  The estimates are fits on one GB300: 512^3 takes 14 us here and 24 on
+// the tensor cores, 640^3 24 on both, 2000 x 2000 x 16 33 here and 23 on either other path.
+template <typename T>
+bool use_small(const Handle *h, const TcPlan &tc, int64_t m, int64_t n, int64_t k, int tri)
+{
+    const double work = (double)m * n * k, part = tri ? 0.5 : 1.0;
+    if (sizeof(T) == 8)
+        return work <= (double)(1ll << 35) && (k > 64 || (double)m * n <= (double)(1 << 24));
+    const double tiles = part * (double)((m + 31) / 32) * ((n + 31) / 32);
+    double small = std::numeric_limits<double>::max();
+    for (int cs = 1; cs <= 8 && (cs == 1 || cs * 64 <= k); cs *= 2)
+        small = std::min(small, 2500 + std::ceil(tiles * cs / h->sms) *
+                                           (400 + 750 * std::ceil((double)k / (64 * cs))) +
+                                    (cs > 1 ? 800 : 0));
+    if (!tc.use) return small < 12000 + 0.00265 * part * m * n + 8e-5 * part * work;
+    const double planes = (double)m * k + (tri ? 0.0 : (double)n * k);
+    return small < 12000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * tc.cost;
 }
 
 // Workspace a call needs: the plan's control words, and the data of whichever path runs (the
@@ -397,22 +421,32 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
 {
     if (h->ws == nullptr) return GFIP_ERR_WORKSPACE;
     ws_limit = std::min(ws_limit, h->ws_bytes);
-    // A workspace too small for the split planes still serves the FFMA path.
-    TcPlan tc = tc_plan<T>(h, m, n, k, tri);
-    if (tc.use) {
-        // The FFMA launch behind it runs only for operands outside the split's range, so the
-        // separate pack pass of pack-then-compute (same bits) is left out.
-        const Variant w = v == Variant::PackThenCompute ? Variant::Direct : v;
-        const Plan<T> behind = make_plan<T>(h, w, (int)m, (int)n, (int)k, tri, tmask_a || tmask_b);
-        tc.use = call_bytes(h, behind, tc) <= ws_limit;
-        if (tc.use) v = w;
-    }
     Plan<T> pl = make_plan<T>(h, v, (int)m, (int)n, (int)k, tri, tmask_a || tmask_b);
     if (total_bytes(h, pl) > ws_limit) return GFIP_ERR_WORKSPACE;
 
     // Grow the control region if this plan needs more of it.
     if (const int rc = grow_ctrl(h, round_up(pl.ctrl_needed, kCtrlGranule)); rc != GFIP_OK)
         return rc;
+
+    // A workspace too small for the split planes still serves the FFMA path.
+    TcPlan tc = tc_plan<T>(h, m, n, k, tri);
+    tc.use = tc.use && call_bytes(h, pl, tc) <= ws_limit;
+    if (use_small<T>(h, tc, m, n, k, tri)) {
+        const gfip::SmallParams<T> sp{A, B, C, lda, ldb, ldc, (int)m, (int)n, (int)k, alpha, beta,
+                                      is_notrans(transa) ? 1 : 0, is_notrans(transb) ? 0 : 1,
+                                      tri, tmask_a, tmask_b, 0, 0};
+        if (gfip::launch_small<T>(sp, h->sms, h->stream, &h->last_grid) != cudaSuccess)
+            return GFIP_ERR_CUDA;
+        h->last_launches = 1;
+        return GFIP_OK;
+    }
+    if (tc.use && v == Variant::PackThenCompute) {
+        // The FFMA launch behind the tensor cores' runs only for operands outside the split's
+        // range: there it reads the operands where they lie (the same bits), and the separate
+        // pack pass is left out.
+        v = Variant::Direct;
+        pl = make_plan<T>(h, v, (int)m, (int)n, (int)k, tri, tmask_a || tmask_b);
+    }
 
     unsigned char *data = h->ws + h->ctrl_bytes;
     gfip::GemmParams<T> p{};

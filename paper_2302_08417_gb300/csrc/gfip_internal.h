@@ -214,6 +214,20 @@ template <typename T> cudaError_t launch_grouped(const GroupParams<T> &gp, cudaS
 // Bytes of one grouped launch's descriptor arrays for `count` problems (element size es).
 size_t grouped_desc_bytes(int count, int es);
 
+// Small products (gfip_small.cu): one launch, no packing, no workspace.  *grid: its CTAs.
+template <typename T> struct SmallParams {
+    const T *A;
+    const T *B;
+    T *C;
+    int64_t lda, ldb, ldc;
+    int m, n, k;
+    T alpha, beta;
+    int a_contig_m, b_contig_n;   // as in GemmParams
+    int tri, tmask_a, tmask_b;    // as in GemmParams
+    int mt, tiles;                // tiles along m, and of C (set by the launcher)
+};
+template <typename T> cudaError_t launch_small(SmallParams<T> p, int sms, cudaStream_t s, int *grid);
+
 // Launchers (defined per element type in gfip_f64.cu / gfip_f32.cu).
 template <typename T> cudaError_t launch_gemm(const GemmParams<T> &p, cudaStream_t s);
 template <typename T> cudaError_t launch_pack(const PackParams<T> &p, cudaStream_t s);

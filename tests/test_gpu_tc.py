@@ -39,8 +39,8 @@ def test_digit_counts_and_chunk_edges(runner, slices):
         assert runner.h.status() == 0
 
 
-@pytest.mark.parametrize("m,n,k", [(128, 128, 128), (129, 257, 130), (64, 300, 255),
-                                   (300, 64, 257), (200, 190, 4001), (1030, 1100, 289)])
+@pytest.mark.parametrize("m,n,k", [(700, 650, 600), (2000, 1500, 16), (1030, 1100, 289),
+                                   (130, 8000, 255), (2100, 129, 1025), (300, 290, 7001)])
 def test_fp32_shapes(runner, m, n, k):
     for ta, tb in (("N", "N"), ("T", "T")):
         p = inputs.problem(m + n + k, ta, tb, m, n, k, -0.75, 0.5, 7, 3, 5, dtype=np.float32)
@@ -57,7 +57,7 @@ def test_fp32_shapes(runner, m, n, k):
 def test_fp32_magnitudes(runner, ea, eb):
     """Operands whose low planes are still normal BF16 numbers, and ones that would leave the
     range: the error bound holds on both sides of the line."""
-    p = inputs.problem(500 + ea, "N", "T", 140, 150, 160, 1.0, 0.0, 3, 1, 2, dtype=np.float32)
+    p = inputs.problem(500 + ea, "N", "T", 700, 680, 660, 1.0, 0.0, 3, 1, 2, dtype=np.float32)
     # magnitudes in [1/2, 1) times the power of two
     p.A, p.B = (np.ldexp(np.copysign(0.5 + np.abs(x) / 2, x), e).astype(np.float32)
                 for x, e in ((p.A, ea), (p.B, eb)))
@@ -69,7 +69,7 @@ def test_fp32_magnitudes(runner, ea, eb):
 def test_fp32_special_operands(runner, value):
     """One infinity, NaN, near-overflow or subnormal entry of A: its row of C has the oracle's
     IEEE classes, every other row is within the bound; and the next call is unaffected."""
-    p = inputs.problem(77, "N", "N", 200, 180, 190, 1.0, 0.0, 0, 0, 0, dtype=np.float32)
+    p = inputs.problem(77, "N", "N", 700, 680, 660, 1.0, 0.0, 0, 0, 0, dtype=np.float32)
     clean = p.A.copy()
     p.A[5 + 17 * p.lda] = value
     got, _ = runner.run(p)
