@@ -288,14 +288,13 @@ struct Group {
     __device__ __forceinline__ int tlo(int s) const { return max(1, c0 - s); }
 };
 
-template <int KIND> __device__ __forceinline__ int group_count(int planes)
+__device__ __forceinline__ int group_count(int planes)
 {
-    return KIND == KIND_F32 ? 1 : (planes + 3) / 4;
+    return (planes + 3) / 4;
 }
 
-template <int KIND> __device__ __forceinline__ Group group_of(int g, int planes)
+__device__ __forceinline__ Group group_of(int g, int planes)
 {
-    if (KIND == KIND_F32) return Group{2, 4, F32_CHUNK_BLOCKS};
     const int c0 = 2 + 4 * g, c1 = min(c0 + 3, planes + 1);
     return Group{c0, c1, EXACT_TERMS / (c1 - 1) / KB};   // a class has at most c1 - 1 pairs
 }
@@ -345,7 +344,14 @@ __device__ __forceinline__ Unit unit_of(const TcParams &p, int u)
     return x;
 }
 
-// Shared-memory slots: `na` A slots used round robin, then `nb` B stages of `planes` slots.
+// FP32: a stage holds a k block's three planes of A, then of B, on one barrier pair (`afull`,
+// `aempty`): its 12 MMAs are issued after a single wait.
+constexpr int F32_PLANES = 3;
+constexpr int F32_STAGES = 4;
+constexpr uint32_t F32_BYTES = F32_PLANES * PLANE_BYTES;
+static_assert(F32_STAGES * 2 * F32_PLANES <= SLOTS && F32_STAGES <= MAX_ASLOTS, "stages fit");
+
+// Digits: `na` A slots used round robin, then `nb` B stages of `planes` slots.
 struct Ring {
     int na, nb;
 };
@@ -359,7 +365,7 @@ __device__ __forceinline__ Ring ring_of(int planes)
 
 // ---- producer -----------------------------------------------------------------------------------
 
-template <int KIND> __device__ void producer(const TcParams &p, Smem &sm)
+__device__ __forceinline__ void digit_producer(const TcParams &p, Smem &sm)
 {
     const Ring rg = ring_of(p.planes);
     const bool leader = elect_one();
@@ -369,11 +375,11 @@ template <int KIND> __device__ void producer(const TcParams &p, Smem &sm)
     bool skip = withhold;   // test hook: the first A plane is never copied
     bool ok = true;
     const int64_t block = (int64_t)p.planes * PLANE_BYTES;
-    const int groups = group_count<KIND>(p.planes);
+    const int groups = group_count(p.planes);
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit x = unit_of(p, u);
         for (int g = 0; g < groups && ok; ++g) {
-            const Group q = group_of<KIND>(g, p.planes);
+            const Group q = group_of(g, p.planes);
             const uint8_t *a = p.pa + ((int64_t)x.i * p.kt + x.kb0) * block;
             const uint8_t *b = p.pb + ((int64_t)x.j * p.kt + x.kb0) * block;
             const uint32_t b_bytes = (q.c1 - 1) * PLANE_BYTES;
@@ -417,11 +423,40 @@ template <int KIND> __device__ void producer(const TcParams &p, Smem &sm)
             mbar_wait_drain(&sm.bfull[i], (i < b_stage ? b_lap : b_lap - 1) & 1u, p.wait_ns);
 }
 
+__device__ __forceinline__ void f32_producer(const TcParams &p, Smem &sm)
+{
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t lap = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+        const Unit x = unit_of(p, u);
+        const uint8_t *a = p.pa + ((int64_t)x.i * p.kt + x.kb0) * F32_BYTES;
+        const uint8_t *b = p.pb + ((int64_t)x.j * p.kt + x.kb0) * F32_BYTES;
+        for (int kb = x.kb0; kb < x.kb1; ++kb, a += F32_BYTES, b += F32_BYTES) {
+            ok = mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
+            if (!ok) break;
+            if (leader) {
+                uint8_t *dst = sm.plane[stage * 2 * F32_PLANES];
+                mbar_expect_tx(&sm.afull[stage], 2 * F32_BYTES);
+                bulk_copy(dst, a, F32_BYTES, &sm.afull[stage]);
+                bulk_copy(dst + F32_BYTES, b, F32_BYTES, &sm.afull[stage]);
+            }
+            if (++stage == F32_STAGES) {
+                stage = 0;
+                ++lap;
+            }
+        }
+    }
+    for (int i = 0; i < F32_STAGES; ++i)   // no copy may outlive the CTA
+        if (i < stage || lap > 0)
+            mbar_wait_drain(&sm.afull[i], (i < stage ? lap : lap - 1) & 1u, p.wait_ns);
+}
+
 // ---- MMA issuer ---------------------------------------------------------------------------------
 
-template <int KIND> __device__ void issuer(const TcParams &p, Smem &sm, uint32_t tmem)
+__device__ __forceinline__ void digit_issuer(const TcParams &p, Smem &sm, uint32_t tmem)
 {
-    constexpr int NBUF = KIND == KIND_F32 ? 2 : 1;
     const Ring rg = ring_of(p.planes);
     const bool leader = elect_one();
     int a_slot = 0, b_stage = 0;
@@ -430,62 +465,44 @@ template <int KIND> __device__ void issuer(const TcParams &p, Smem &sm, uint32_t
     bool ok = true;
     const uint32_t a_base = desc_low(saddr(sm.plane[0]));
     const uint32_t b_base = a_base + rg.na * PLANE_DESC;
-    const int groups = group_count<KIND>(p.planes);
+    const int groups = group_count(p.planes);
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit x = unit_of(p, u);
         for (int g = 0; g < groups && ok; ++g) {
-            const Group q = group_of<KIND>(g, p.planes);
+            const Group q = group_of(g, p.planes);
             for (int k0 = x.kb0; k0 < x.kb1 && ok; k0 += q.chunk, ++chunks) {
                 const int k1 = min(x.kb1, k0 + q.chunk);
-                const int buf = chunks % NBUF;
-                ok = mbar_wait(&sm.tempty[buf], ((chunks / NBUF) & 1u) ^ 1u, sm, p.status,
-                               p.wait_ns);
+                ok = mbar_wait(&sm.tempty[0], (chunks & 1u) ^ 1u, sm, p.status, p.wait_ns);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d0 = tmem + buf * 256;
                 uint32_t accumulate = 0;   // the first A plane's products start the sums
                 for (int kb = k0; kb < k1; ++kb) {
                     ok = mbar_wait(&sm.bfull[b_stage], b_phase, sm, p.status, p.wait_ns);
                     if (!ok) break;
                     const uint32_t b1 = b_base + b_stage * p.planes * PLANE_DESC;
-                    auto step = [&](auto &&mmas) -> bool {
-                        if (!mbar_wait(&sm.afull[a_slot], a_phase, sm, p.status, p.wait_ns))
-                            return false;
+                    for (int s = 1; s < q.c1; ++s) {
+                        ok = mbar_wait(&sm.afull[a_slot], a_phase, sm, p.status, p.wait_ns);
+                        if (!ok) break;
                         tc_fence_after();
                         if (leader) {
-                            mmas(a_base + a_slot * PLANE_DESC);
+                            const int lo = q.tlo(s);
+                            const uint32_t a = a_base + a_slot * PLANE_DESC;
+                            uint32_t b = b1 + (lo - 1) * PLANE_DESC;
+                            uint32_t d = tmem + (s + lo - q.c0) * TN;
+                            int left = q.c1 - s - lo + 1;
+                            for (; left >= 2; left -= 2) {
+                                mma_block<256>(d, a, b, accumulate);
+                                b += 2 * PLANE_DESC;
+                                d += 2 * TN;
+                            }
+                            if (left) mma_block<128>(d, a, b, accumulate);
                             mma_commit(&sm.aempty[a_slot]);
                         }
+                        accumulate = 1;
                         if (++a_slot == rg.na) {
                             a_slot = 0;
                             a_phase ^= 1u;
                         }
-                        accumulate = 1;
-                        return true;
-                    };
-                    if constexpr (KIND == KIND_F32) {
-                        // columns 0-127: a1 b1; 128-255: the five smaller products
-                        ok = step([&](uint32_t a) {
-                            mma_block<256>(d0, a, b1, accumulate);
-                            mma_block<128>(d0 + TN, a, b1 + 2 * PLANE_DESC, 1u);
-                        }) && step([&](uint32_t a) {
-                            mma_block<128>(d0 + TN, a, b1, 1u);
-                            mma_block<128>(d0 + TN, a, b1 + PLANE_DESC, 1u);
-                        }) && step([&](uint32_t a) { mma_block<128>(d0 + TN, a, b1, 1u); });
-                    } else {
-                        for (int s = 1; s < q.c1 && ok; ++s)
-                            ok = step([&](uint32_t a) {
-                                const int lo = q.tlo(s);
-                                uint32_t b = b1 + (lo - 1) * PLANE_DESC;
-                                uint32_t d = d0 + (s + lo - q.c0) * TN;
-                                int left = q.c1 - s - lo + 1;
-                                for (; left >= 2; left -= 2) {
-                                    mma_block<256>(d, a, b, accumulate);
-                                    b += 2 * PLANE_DESC;
-                                    d += 2 * TN;
-                                }
-                                if (left) mma_block<128>(d, a, b, accumulate);
-                            });
                     }
                     if (!ok) break;
                     if (leader) mma_commit(&sm.bempty[b_stage]);
@@ -494,8 +511,55 @@ template <int KIND> __device__ void issuer(const TcParams &p, Smem &sm, uint32_t
                         b_phase ^= 1u;
                     }
                 }
-                if (ok && leader) mma_commit(&sm.tfull[buf]);
+                if (ok && leader) mma_commit(&sm.tfull[0]);
             }
+        }
+    }
+    // all MMAs this warp issued have completed once this commit arrives
+    if (leader) mma_commit(&sm.drain);
+    mbar_wait_drain(&sm.drain, 0, p.wait_ns);
+}
+
+__device__ __forceinline__ void f32_issuer(const TcParams &p, Smem &sm, uint32_t tmem)
+{
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0, chunks = 0;
+    bool ok = true;
+    const uint32_t base = desc_low(saddr(sm.plane[0]));
+    for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+        const Unit x = unit_of(p, u);
+        for (int k0 = x.kb0; k0 < x.kb1 && ok; k0 += F32_CHUNK_BLOCKS, ++chunks) {
+            const int k1 = min(x.kb1, k0 + F32_CHUNK_BLOCKS);
+            const uint32_t buf = chunks & 1u;
+            ok = mbar_wait(&sm.tempty[buf], ((chunks >> 1) & 1u) ^ 1u, sm, p.status, p.wait_ns);
+            if (!ok) break;
+            tc_fence_after();
+            // columns 0-127: a1 b1; 128-255: the five smaller products
+            const uint32_t d = tmem + buf * 256;
+            uint32_t accumulate = 0;   // the block's first MMA starts both sums
+            for (int kb = k0; kb < k1; ++kb) {
+                ok = mbar_wait(&sm.afull[stage], phase, sm, p.status, p.wait_ns);
+                if (!ok) break;
+                tc_fence_after();
+                if (leader) {
+                    const uint32_t a1 = base + stage * 2 * F32_PLANES * PLANE_DESC;
+                    const uint32_t a2 = a1 + PLANE_DESC, a3 = a2 + PLANE_DESC;
+                    const uint32_t b1 = a3 + PLANE_DESC, b2 = b1 + PLANE_DESC;
+                    mma_block<256>(d, a1, b1, accumulate);
+                    mma_block<128>(d + TN, a1, b2 + PLANE_DESC, 1u);
+                    mma_block<128>(d + TN, a2, b1, 1u);
+                    mma_block<128>(d + TN, a2, b2, 1u);
+                    mma_block<128>(d + TN, a3, b1, 1u);
+                    mma_commit(&sm.aempty[stage]);
+                }
+                accumulate = 1;
+                if (++stage == F32_STAGES) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+            if (ok && leader) mma_commit(&sm.tfull[buf]);
         }
     }
     // all MMAs this warp issued have completed once this commit arrives
@@ -505,6 +569,12 @@ template <int KIND> __device__ void issuer(const TcParams &p, Smem &sm, uint32_t
 
 // ---- epilogue -----------------------------------------------------------------------------------
 
+// x * 2^e where the result or x is zero, subnormal or not finite.
+[[maybe_unused]] static __device__ __noinline__ double scale2_general(double x, int e)
+{
+    return ldexp(x, e);
+}
+
 // x * 2^e; the fast path adds to the exponent field.
 __device__ __forceinline__ double scale2(double x, int e)
 {
@@ -512,7 +582,7 @@ __device__ __forceinline__ double scale2(double x, int e)
     const int ex = ((hi >> 20) & 0x7FF) + e;
     if (((hi >> 20) & 0x7FF) != 0 && ex > 0 && ex < 2047)
         return __hiloint2double(hi + e * (1 << 20), __double2loint(x));
-    return ldexp(x, e);
+    return scale2_general(x, e);
 }
 
 template <int KIND> struct AccOf {
@@ -568,15 +638,31 @@ template <int KIND> __device__ void epilogue(const TcParams &p, Smem &sm, uint32
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tensor-memory lane quarter from warp % 4, column half from (warp - 2) / 4
     const int quarter = warp & 3, half = (warp - 2) >> 2;
-    const int groups = group_count<KIND>(p.planes);
+    const int groups = KIND == KIND_F32 ? 1 : group_count(p.planes);
     uint32_t chunks = 0;
     for (int u = blockIdx.x; u < p.units; u += gridDim.x) {
         const Unit x = unit_of(p, u);
+        const int row = x.i * TM + quarter * 32 + lane;
+        const int col0 = x.j * TN + half * 64;
+        T *C = static_cast<T *>(p.C);
+        const T alpha = (T)p.alpha, beta = (T)p.beta;
+        const bool read_c = beta != T(0);
+        // bring C to L2 while the products are formed: lane l fetches columns l and l + 32 of
+        // the warp's 32 rows (128 bytes of FP32, 256 of FP64)
+        if (read_c) {
+            const int row0 = row - lane;
+            for (int c = lane; c < 64; c += 32)
+                if (col0 + c < p.n)
+                    for (int r = row0; r < min(row0 + 32, p.m); r += 128 / (int)sizeof(T))
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(
+                            C + r + (int64_t)(col0 + c) * p.ldc));
+        }
         Acc acc[64];
 #pragma unroll
         for (int c = 0; c < 64; ++c) acc[c] = Acc(0);
         for (int g = 0; g < groups; ++g) {
-            const Group q = group_of<KIND>(g, p.planes);
+            const Group q =
+                KIND == KIND_F32 ? Group{2, 4, F32_CHUNK_BLOCKS} : group_of(g, p.planes);
             for (int k0 = x.kb0; k0 < x.kb1; k0 += q.chunk, ++chunks) {
                 const int buf = chunks % NBUF;
                 if (!mbar_wait(&sm.tfull[buf], (chunks / NBUF) & 1u, sm, p.status, p.wait_ns))
@@ -616,11 +702,6 @@ template <int KIND> __device__ void epilogue(const TcParams &p, Smem &sm, uint32
                 if (lane == 0) mbar_arrive(&sm.tempty[buf]);
             }
         }
-        const int row = x.i * TM + quarter * 32 + lane;
-        const int col0 = x.j * TN + half * 64;
-        T *C = static_cast<T *>(p.C);
-        const T alpha = (T)p.alpha, beta = (T)p.beta;
-        const bool read_c = beta != T(0);
         if constexpr (KIND == KIND_F32) {
             if (p.splits > 1) {
                 // every split stores its partial tile; of each warp's 32 x 64 part the last to
@@ -653,33 +734,41 @@ template <int KIND> __device__ void epilogue(const TcParams &p, Smem &sm, uint32
             er = p.ea[row] + 2;   // 2^(e_i + 1) 2^(f_j + 1)
             if (KIND == KIND_DIGITS_INT) er -= DIGIT_BITS * (p.planes + 1);
         }
+        // The columns this row stores: up to n, and of a triangle the row's part.  (Code that
+        // decides per column runs at the rate of instruction fetches: 64 columns of it took
+        // 25000 clocks a tile at 2048^3.)
+        const int first = p.tri == TRI_UPPER ? row : 0;
+        const int end = p.tri == TRI_LOWER ? min(p.n, row + 1) : p.n;
+        const uint32_t count = end > first ? static_cast<uint32_t>(end - first) : 0u;
         // C is read W columns at a time, before any of them is written
-        constexpr int W = KIND == KIND_F32 ? 16 : 8;
+        constexpr int W = KIND == KIND_F32 ? 32 : 8;
+        T *cp = C + row + (int64_t)col0 * p.ldc;
+        const T *cr = cp;
 #pragma unroll
         for (int g = 0; g < 64 / W; ++g) {
             T cv[W];
-            bool in[W];
+            if (read_c) {
 #pragma unroll
-            for (int i = 0; i < W; ++i) {
-                const int col = col0 + g * W + i;
-                in[i] = col < p.n;
-                if (p.tri == TRI_LOWER) in[i] = in[i] && row >= col;
-                if (p.tri == TRI_UPPER) in[i] = in[i] && row <= col;
-                cv[i] = (read_c && in[i]) ? C[row + (int64_t)col * p.ldc] : T(0);
+                for (int i = 0; i < W; ++i) {
+                    cv[i] = T(0);
+                    if (static_cast<uint32_t>(col0 + g * W + i - first) < count) cv[i] = *cr;
+                    cr += p.ldc;
+                }
             }
 #pragma unroll
             for (int i = 0; i < W; ++i) {
                 const int col = col0 + g * W + i;
-                if (!in[i]) continue;
+                const bool in = static_cast<uint32_t>(col - first) < count;
                 T v;
                 if constexpr (KIND == KIND_F32) {
                     v = alpha * acc[g * W + i];
                     if (read_c) v = fmaf(beta, cv[i], v);
                 } else {
-                    v = alpha * scale2((double)acc[g * W + i], er + p.eb[col]);
+                    v = alpha * scale2((double)acc[g * W + i], er + (in ? p.eb[col] : 0));
                     if (read_c) v = fma(beta, cv[i], v);
                 }
-                C[row + (int64_t)col * p.ldc] = v;
+                if (in) *cp = v;
+                cp += p.ldc;
             }
         }
     }
@@ -726,9 +815,11 @@ template <int KIND> __global__ void __launch_bounds__(THREADS, 1) tc_kernel(cons
     const uint32_t tmem = sm.tmem_base;
 
     if (warp == 0) {
-        producer<KIND>(p, sm);
+        if constexpr (KIND == KIND_F32) f32_producer(p, sm);
+        else digit_producer(p, sm);
     } else if (warp == 1) {
-        issuer<KIND>(p, sm, tmem);
+        if constexpr (KIND == KIND_F32) f32_issuer(p, sm, tmem);
+        else digit_issuer(p, sm, tmem);
     } else {
         epilogue<KIND>(p, sm, tmem);
     }
