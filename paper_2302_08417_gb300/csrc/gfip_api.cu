@@ -778,9 +778,11 @@ size_t trsm_workspace_min(Handle *h, char side, int64_t m, int64_t n)
     // workspace grows with each dimension
     const bool left = side == 'L' || side == 'l';
     const int na = (int)(left ? m : n);
-    const Plan<T> panel =
-        make_plan<T>(h, Variant::Fused, (int)m, (int)n, std::min(gfip::TRSM_PANEL, na));
-    return total_bytes(h, panel);
+    const int pw = std::min(gfip::TRSM_PANEL, na);
+    const Plan<T> panel = make_plan<T>(h, Variant::Fused, (int)m, (int)n, pw);
+    // (a panel's packed triangle, FP32, is smaller than the plan's partial tiles or panels)
+    return std::max(total_bytes(h, panel),
+                    h->ctrl_bytes + (sizeof(T) == 4 ? gfip::trsm_image_bytes(pw) : 0));
 }
 
 // ... and with room for the tensor-core path of the updates that take it.
@@ -867,11 +869,20 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
         const int p0 = pi * gfip::TRSM_PANEL;
         const int pw = std::min(gfip::TRSM_PANEL, na - p0);
         // the panel's unknowns: rows p0.. of B (side L) or its columns p0.. (side R)
-        const cudaError_t e =
-            left ? gfip::launch_trsm_panel<T>(B + p0, ldb, 1, (int)n, A, lda, trans, p0, pw,
-                                              lower_t, 0, unit, h->stream)
-                 : gfip::launch_trsm_panel<T>(B + (int64_t)p0 * ldb, 1, ldb, (int)m, A, lda,
-                                              trans, p0, pw, lower_t, 1, unit, h->stream);
+        T *Bp = left ? B + p0 : B + (int64_t)p0 * ldb;
+        const int64_t vstride = left ? ldb : 1, estride = left ? 1 : ldb;
+        const int nvec = (int)(left ? n : m);
+        cudaError_t e;
+        if constexpr (sizeof(T) == 4) {
+            // the packed triangle takes the bytes the update's GEMM uses afterwards
+            e = gfip::launch_trsm_panel_f32(Bp, vstride, estride, nvec, A, lda, trans, p0, pw,
+                                            lower_t, left ? 0 : 1, unit,
+                                            reinterpret_cast<float *>(h->ws + h->ctrl_bytes),
+                                            reinterpret_cast<unsigned int *>(h->ws), h->stream);
+        } else {
+            e = gfip::launch_trsm_panel_f64(Bp, vstride, estride, nvec, A, lda, trans, p0, pw,
+                                            lower_t, left ? 0 : 1, unit, h->stream);
+        }
         if (e != cudaSuccess) return GFIP_ERR_CUDA;
         const int rc = lower_t ? update(p0, pw, p0 + pw, na) : update(p0, pw, 0, p0);
         if (rc != GFIP_OK) return rc;

@@ -1,4 +1,5 @@
-// gfip_trsm.cu -- the panel solves of the blocked triangular solve (TRSM).
+// gfip_trsm.cu -- the panel solves of the blocked triangular solve (TRSM) in FP64 (FP32:
+// gfip_trsm_f32.cu).
 //
 // TRSM runs as a sequence over panels of op(A)'s diagonal (see gfip_api.cu): each step solves
 // one panel of at most TRSM_PANEL unknowns for every right-hand side with the kernel below,
@@ -6,8 +7,8 @@
 // solved.  The kernel solves a panel by column-oriented substitution: once unknown d is known
 // (divided by its diagonal entry), every unknown below it loses its multiple at once; per
 // chunk of columns the chain updates only its own 32-row group, and the later groups are
-// updated afterwards, off the chain.  A warp holds one or two right-hand sides, one element
-// per lane and 32-row group, in registers; the panel's triangle streams through shared memory
+// updated afterwards, off the chain.  A warp holds one right-hand side, one element per lane
+// and 32-row group, in registers; the panel's triangle streams through shared memory
 // in chunks of columns, double-buffered and shared by the CTA's warps, the next chunk loaded
 // into registers while this one is solved.  Only the entries a triangular solve reads are
 // read: never the other triangle, nor a unit diagonal.
@@ -18,14 +19,12 @@
 namespace gfip {
 namespace trsm {
 
-// Right-hand sides per warp: FP32 two (8 warps a CTA: the two chains interleave within the
-// warp; 6 % faster at 2048 x 2048 than one a warp in 16 warps), FP64 one (its registers do
-// not hold two, and it is bound by its DFMA pipe): the shortest chain per right-hand side.
-// FP64 runs between 8 and 16 warps a CTA, as many as spread the right-hand sides over all SMs
-// (2048 of them on 152 SMs: 14 a CTA, 147 CTAs, 11 % faster than 16 a CTA on 128 SMs).
+// One right-hand side per warp (the shortest chain per side; the DFMA pipe is the bound), and
+// between 8 and 16 warps a CTA, as many as spread the right-hand sides over all SMs (2048 of
+// them on 152 SMs: 14 a CTA, 147 CTAs, 11 % faster than 16 a CTA on 128 SMs).
 template <typename T> struct Shape {
-    static constexpr int RPW = sizeof(T) == 4 ? 2 : 1;
-    static constexpr int MIN_WARPS = 8 / RPW, MAX_WARPS = 16 / RPW;
+    static constexpr int RPW = 1;
+    static constexpr int MIN_WARPS = 8, MAX_WARPS = 16;
     // staging slots a thread takes per half chunk: one with 512 threads, more with fewer
     // (the kernel is compiled for each)
     static constexpr int MAX_SLOTS = TRSM_PANEL / (MIN_WARPS * 32);
@@ -43,20 +42,11 @@ template <typename T> __host__ __device__ constexpr size_t buf_elems() { return 
 // two chunk buffers, two diagonals and two reciprocal diagonals
 template <typename T> constexpr size_t smem_bytes() { return sizeof(T) * (2 * buf_elems<T>() + 4 * CW); }
 
-// 16-byte shared-memory accesses of a row (float4 / double2)
-__device__ __forceinline__ void ld16(const float *s, float (&v)[4])
-{
-    const float4 t = *reinterpret_cast<const float4 *>(s);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
+// 16-byte shared-memory accesses of a row
 __device__ __forceinline__ void ld16(const double *s, double (&v)[2])
 {
     const double2 t = *reinterpret_cast<const double2 *>(s);
     v[0] = t.x; v[1] = t.y;
-}
-__device__ __forceinline__ void st16(float *s, const float *v)
-{
-    *reinterpret_cast<float4 *>(s) = make_float4(v[0], v[1], v[2], v[3]);
 }
 __device__ __forceinline__ void st16(double *s, const double *v)
 {
@@ -214,7 +204,7 @@ __global__ void __launch_bounds__(Shape<T>::MAX_WARPS * 32, 1)
     panel_kernel(T *B, int64_t vstride, int64_t estride, int nvec, const Panel p)
 {
     constexpr int RPW = Shape<T>::RPW;
-    constexpr int PADW = padw<T>(), V = 16 / (int)sizeof(T);
+    constexpr int PADW = padw<T>();
     constexpr size_t BUF = buf_elems<T>();
     const int rpc = (blockDim.x >> 5) * RPW;   // right-hand sides of this CTA
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -277,78 +267,24 @@ __global__ void __launch_bounds__(Shape<T>::MAX_WARPS * 32, 1)
             Stage<T, SLOTS> st;
             if (more) stage_load<T, SLOTS>(p, d0 + CW, 0, tid, st);
             const int dn = min(CW, pw - d0);
-            // this lane's row of the chunk (its entries left of the diagonal: FP32 reads it
-            // whole ahead of the chain, FP64, short of registers, an entry a step), and, for
-            // the lane whose unknown is in the chunk, its diagonal entry and reciprocal
+            // this lane's row of the chunk, and, for the lane whose unknown is in the chunk, its
+            // diagonal entry and reciprocal
             const int ln = lane - h * CW;   // this lane's unknown within the chunk, if in range
             const T *crow = lrow + 32 * r * PADW;
-            constexpr bool PRELOAD = sizeof(T) == 4;
-            T trow[CW];
-            if (PRELOAD) {
-#pragma unroll
-                for (int d4 = 0; d4 < CW; d4 += V) {
-                    T v[V];
-                    ld16(crow + d4, v);
-#pragma unroll
-                    for (int j = 0; j < V; ++j) trow[d4 + j] = v[j];
-                }
-            }
-            const bool inch = ln >= 0 && ln < CW;
             const int lc = ln < 0 ? 0 : (ln >= CW ? CW - 1 : ln);
             const T t = dg[lc], rt = dr[lc];
             // the chunk's unknowns one after another; each updates only the later unknowns
             // of its own 32-row group here (the chain's latency is the solve's floor).
-            // A whole chunk first takes the short form: every lane forms the quotient of its
-            // own element (by its own diagonal entry; lanes outside the chunk, and a unit
-            // diagonal, by 1), the owner's is broadcast, and every lane subtracts its multiple
-            // with its row's entry, which is zero on and above the diagonal, so that the
-            // chunk's unknowns keep their last right-hand side and take their quotient once
-            // the chunk is done (the one the owner broadcast: the same operands).  A
-            // non-finite quotient in any lane makes the chunk run again in the exact form
-            // below (owner-only quotients, the division for special values), as does a short
-            // last chunk.  With finite values both forms give the same bits.  FP64 keeps the
-            // exact form: its extra multiply-adds would load the DFMA pipe that bounds it.
-            bool exact = sizeof(T) == 8 || dn < CW;
-            if (!exact) {
-                const T tl = inch ? t : T(1), rl = inch ? rt : T(1);
-                T cur0[RPW];
-                T acc = T(0);   // stays zero while every quotient is finite
 #pragma unroll
-                for (int w = 0; w < RPW; ++w) cur0[w] = cur[w];
+            for (int dd = 0; dd < CW; ++dd) {
+                if (dd >= dn) break;
 #pragma unroll
-                for (int dd = 0; dd < CW; ++dd)
-#pragma unroll
-                    for (int w = 0; w < RPW; ++w) {
-                        const T q0 = cur[w] * rl;
-                        const T qv = fma(fma(-tl, q0, cur[w]), rl, q0);
-                        acc = fma(qv, T(0), acc);
-                        const T x = __shfl_sync(0xffffffffu, qv, h * CW + dd);
-                        cur[w] = fma(-(PRELOAD ? trow[dd] : crow[dd]), x, cur[w]);
-                    }
-                if (__any_sync(0xffffffffu, !(acc == T(0)))) {
-                    exact = true;
-#pragma unroll
-                    for (int w = 0; w < RPW; ++w) cur[w] = cur0[w];
-                } else if (inch) {
-#pragma unroll
-                    for (int w = 0; w < RPW; ++w) {
-                        const T q0 = cur[w] * rl;
-                        cur[w] = fma(fma(-tl, q0, cur[w]), rl, q0);
-                    }
-                }
-            }
-            if (exact) {
-#pragma unroll
-                for (int dd = 0; dd < CW; ++dd) {
-                    if (dd >= dn) break;
-#pragma unroll
-                    for (int w = 0; w < RPW; ++w) {
-                        T bc = cur[w];
-                        if (!p.unit && ln == dd) bc = quotient(bc, t, rt);
-                        const T x = __shfl_sync(0xffffffffu, bc, h * CW + dd);
-                        if (ln == dd) cur[w] = x;
-                        if (ln > dd) cur[w] = fma(-(PRELOAD ? trow[dd] : crow[dd]), x, cur[w]);
-                    }
+                for (int w = 0; w < RPW; ++w) {
+                    T bc = cur[w];
+                    if (!p.unit && ln == dd) bc = quotient(bc, t, rt);
+                    const T x = __shfl_sync(0xffffffffu, bc, h * CW + dd);
+                    if (ln == dd) cur[w] = x;
+                    if (ln > dd) cur[w] = fma(-crow[dd], x, cur[w]);
                 }
             }
             if (more) {
@@ -447,9 +383,8 @@ cudaError_t launch_trsm_panel_impl(T *B, int64_t vstride, int64_t estride, int n
         if (sms <= 0) sms = 1;
     }
     const int want = (nvec + sms * S::RPW - 1) / (sms * S::RPW);
-    const int warps = sizeof(T) == 4 ? S::MAX_WARPS
-                      : want < S::MIN_WARPS ? S::MIN_WARPS
-                                            : (want > S::MAX_WARPS ? S::MAX_WARPS : want);
+    const int warps = want < S::MIN_WARPS ? S::MIN_WARPS
+                                          : (want > S::MAX_WARPS ? S::MAX_WARPS : want);
     const int rpc = warps * S::RPW;
     const int blocks = (nvec + rpc - 1) / rpc;
     if (warps * 32 >= TRSM_PANEL)
@@ -464,22 +399,12 @@ cudaError_t launch_trsm_panel_impl(T *B, int64_t vstride, int64_t estride, int n
     return cudaGetLastError();
 }
 
-template <>
-cudaError_t launch_trsm_panel<double>(double *B, int64_t vstride, int64_t estride, int nvec,
-                                      const double *A, int64_t lda, int a_trans, int k0, int pw,
-                                      int lower_t, int transpose_t, int unit, cudaStream_t s)
+cudaError_t launch_trsm_panel_f64(double *B, int64_t vstride, int64_t estride, int nvec,
+                                  const double *A, int64_t lda, int a_trans, int k0, int pw,
+                                  int lower_t, int transpose_t, int unit, cudaStream_t s)
 {
     return launch_trsm_panel_impl<double>(B, vstride, estride, nvec, A, lda, a_trans, k0, pw,
                                           lower_t, transpose_t, unit, s);
-}
-
-template <>
-cudaError_t launch_trsm_panel<float>(float *B, int64_t vstride, int64_t estride, int nvec,
-                                     const float *A, int64_t lda, int a_trans, int k0, int pw,
-                                     int lower_t, int transpose_t, int unit, cudaStream_t s)
-{
-    return launch_trsm_panel_impl<float>(B, vstride, estride, nvec, A, lda, a_trans, k0, pw,
-                                         lower_t, transpose_t, unit, s);
 }
 
 }  // namespace gfip
