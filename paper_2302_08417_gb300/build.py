@@ -20,7 +20,8 @@ PROBE = os.path.join(OUT, "peak_probe")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 LIB_SOURCES = ["gfip_api.cu", "gfip_f64.cu", "gfip_f32.cu", "gfip_f32_ws.cu", "gfip_f64_tmask.cu",
-               "gfip_f32_tmask.cu", "gfip_f32_tc.cu", "gfip_small.cu", "gfip_ozaki.cu", "gfip_grouped.cu", "gfip_trsm.cu",
+               "gfip_f32_tmask.cu", "gfip_f32_tc.cu", "gfip_f32_skinny.cu",
+               "gfip_small.cu", "gfip_ozaki.cu", "gfip_grouped.cu", "gfip_trsm.cu",
                "gfip_trsm_f32.cu"]
 HEADERS = ["gfip_internal.h", "gfip_kernels.cuh", "gfip_ws.cuh", "gfip_grouped.h",
            "gfip_testing.h", "gfip_tc.cuh"]

@@ -248,11 +248,15 @@ struct TcPlan {
     bool use = false;
     int mt = 0, nt = 0, kt = 0, tiles = 0, splits = 1;
     int64_t cost = 0;   // k blocks in a row on the busiest SM, overheads counted as blocks
+    double ns = 0;      // estimated time
     size_t off_a = 0, off_b = 0, off_partial = 0, off_counter = 0, data_bytes = 0;
+    bool skinny = false;   // at most 128 rows or columns: gfip_f32_skinny.cu
+    int n16 = 0;           // ... and the small operand's rows, a multiple of 16
 };
 
 template <typename T>
-TcPlan tc_plan(const Handle *h, int64_t m, int64_t n, int64_t k, int tri)
+TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, int64_t k, int tri,
+               bool masked = false)
 {
     TcPlan t;
     if (sizeof(T) != 4 || k > kTcMaxK || k < kTcMinK) return t;
@@ -272,9 +276,27 @@ TcPlan tc_plan(const Handle *h, int64_t m, int64_t n, int64_t k, int tri)
             t.splits = s;
         }
     }
+    // Estimated times, ns, fitted to one GB300: 2048^3 87 us, 64 x 8192 x 8192 205 (its planes' 10
+    // bytes an element dominate) and, split on the way, 112; 100 x 2000 x 2000 29 and 37.
+    const double planes = (double)m * k + (tri ? 0.0 : (double)n * k);
+    const double part = tri ? 0.5 : 1.0;
+    t.ns = 12000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost;
+    // at most 128 rows or columns against an operand that is read along memory
+    if (tri == gfip::TRI_NONE && !masked && std::min(m, n) <= 128 &&
+        (n <= m ? is_notrans(transa) : !is_notrans(transb)) && 14000 + 700.0 * t.cost < t.ns) {
+        t.skinny = true;
+        t.n16 = static_cast<int>((std::min(m, n) + 15) / 16 * 16);
+        t.ns = 14000 + 700.0 * t.cost;
+    }
     const size_t plane = 128 * 32 * 2;
     size_t d = 0;
     t.off_a = d;
+    if (t.skinny) {   // planes of the small operand, partial sums of every unit
+        d += (size_t)3 * t.kt * plane;
+        t.off_partial = d;
+        t.data_bytes = d + (size_t)t.tiles * t.splits * t.n16 * 128 * sizeof(float);
+        return t;
+    }
     d += (size_t)3 * t.mt * t.kt * plane;
     t.off_b = tri ? t.off_a : d;
     if (!tri) d += (size_t)3 * t.nt * t.kt * plane;
@@ -309,8 +331,7 @@ bool use_small(const Handle *h, const TcPlan &tc, int64_t m, int64_t n, int64_t 
                                            (400 + 750 * std::ceil((double)k / (64 * cs))) +
                                     (cs > 1 ? 800 : 0));
     if (!tc.use) return small < 12000 + 0.00265 * part * m * n + 8e-5 * part * work;
-    const double planes = (double)m * k + (tri ? 0.0 : (double)n * k);
-    return small < 12000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * tc.cost;
+    return small < tc.ns;
 }
 
 // Workspace a call needs: the plan's control words, and the data of whichever path runs (the
@@ -382,6 +403,33 @@ int gemm_entry(gfip_handle_t handle, Variant v, char transa, char transb, int64_
 cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<float> &p,
                       unsigned char *data)
 {
+    if (t.skinny) {
+        const bool big_is_row = p.n <= p.m;   // op(A) is the large operand
+        gfip::SkinnyParams q{};
+        q.X = big_is_row ? p.A : p.B;
+        q.ld = big_is_row ? p.lda : p.ldb;
+        q.rows = big_is_row ? p.m : p.n;
+        q.k = p.k;
+        q.planes = data + t.off_a;
+        q.n16 = t.n16;
+        q.kt = t.kt;
+        q.tiles = t.tiles;
+        q.splits = t.splits;
+        q.units = t.tiles * t.splits;
+        q.partial = reinterpret_cast<float *>(data + t.off_partial);
+        q.gate = p.gate;
+        q.status = p.status;
+        q.wait_ns = kOzakiWaitNs;
+        const gfip::F32SplitArgs small{big_is_row ? p.B : p.A,
+                                       big_is_row ? p.ldb : p.lda,
+                                       big_is_row ? p.n : p.m,
+                                       big_is_row ? p.b_contig_n : p.a_contig_m,
+                                       1,
+                                       0,
+                                       data + t.off_a};
+        return gfip::launch_f32_skinny(q, small, p.C, p.ldc, big_is_row ? 1 : 0, p.alpha, p.beta,
+                                       h->sms, h->stream);
+    }
     gfip::TcParams q{};
     q.pa = data + t.off_a;
     q.pb = data + t.off_b;
@@ -429,7 +477,7 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
         return rc;
 
     // A workspace too small for the split planes still serves the FFMA path.
-    TcPlan tc = tc_plan<T>(h, m, n, k, tri);
+    TcPlan tc = tc_plan<T>(h, transa, transb, m, n, k, tri, tmask_a || tmask_b);
     tc.use = tc.use && call_bytes(h, pl, tc) <= ws_limit;
     if (use_small<T>(h, tc, m, n, k, tri)) {
         const gfip::SmallParams<T> sp{A, B, C, lda, ldb, ldc, (int)m, (int)n, (int)k, alpha, beta,
@@ -503,7 +551,7 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
         if (tc.use) {
             p.gate = reinterpret_cast<unsigned int *>(h->ws + kGateOffset);
             if (launch_tc(h, tc, p, data) != cudaSuccess) return GFIP_ERR_CUDA;
-            launches += 2;
+            launches += tc.skinny ? 3 : 2;
         }
     }
     if (v == Variant::PackThenCompute) {
@@ -605,7 +653,7 @@ size_t workspace_size_impl(Handle *h, char transa, char transb, int64_t m, int64
     if (too_big(m) || too_big(n) || too_big(k)) return 0;
     if (m == 0 || n == 0 || k == 0) return round_up(kHeader, kCtrlGranule);
     const Plan<T> pl = make_plan<T>(h, v, (int)m, (int)n, (int)k);
-    return call_bytes(h, pl, tc_plan<T>(h, m, n, k, gfip::TRI_NONE));
+    return call_bytes(h, pl, tc_plan<T>(h, transa, transb, m, n, k, gfip::TRI_NONE));
 }
 
 // Reference-BLAS dsyrk argument check: 0, or minus the 1-based position of the first bad
@@ -669,7 +717,7 @@ size_t syrk_workspace_impl(Handle *h, char uplo, char trans, int64_t n, int64_t 
     if (n == 0 || k == 0) return round_up(kHeader, kCtrlGranule);
     const int tri = (uplo == 'L' || uplo == 'l') ? gfip::TRI_LOWER : gfip::TRI_UPPER;
     const Plan<T> pl = make_plan<T>(h, Variant::Fused, (int)n, (int)n, (int)k, tri);
-    return call_bytes(h, pl, tc_plan<T>(h, n, n, k, tri));
+    return call_bytes(h, pl, tc_plan<T>(h, 'N', 'T', n, n, k, tri));
 }
 
 // Reference-BLAS dtrmm argument check: 0, or minus the 1-based position of the first bad
@@ -710,7 +758,7 @@ size_t trmm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
     const bool left = side == 'L' || side == 'l';
     const Plan<T> pl =
         make_plan<T>(h, Variant::Fused, (int)m, (int)n, (int)(left ? m : n), gfip::TRI_NONE, true);
-    const TcPlan tc = tc_plan<T>(h, m, n, left ? m : n, gfip::TRI_NONE);
+    const TcPlan tc = tc_plan<T>(h, 'N', 'N', m, n, left ? m : n, gfip::TRI_NONE, true);
     return round_up(call_bytes(h, pl, tc), kAlign) + round_up((size_t)m * n * sizeof(T), kAlign);
 }
 
@@ -748,7 +796,7 @@ int trmm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     const size_t w_bytes = (size_t)m * n * sizeof(T);
     // a workspace without room for the split planes of the tensor-core path runs without it
     size_t w_off =
-        round_up(call_bytes(h, pl, tc_plan<T>(h, m, n, kdim, gfip::TRI_NONE)), kAlign);
+        round_up(call_bytes(h, pl, tc_plan<T>(h, 'N', 'N', m, n, kdim, gfip::TRI_NONE, true)), kAlign);
     if (w_off + w_bytes > h->ws_bytes) w_off = round_up(total_bytes(h, pl), kAlign);
     if (w_off + w_bytes > h->ws_bytes) return GFIP_ERR_WORKSPACE;
     T *W = reinterpret_cast<T *>(h->ws + w_off);
@@ -796,8 +844,9 @@ size_t trsm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
         auto update = [&](int64_t rest, int64_t width) {
             const int64_t um = left ? rest : m, un = left ? n : rest;
             const Plan<T> pl = make_plan<T>(h, Variant::Fused, (int)um, (int)un, (int)width);
-            bytes =
-                std::max(bytes, call_bytes(h, pl, tc_plan<T>(h, um, un, width, gfip::TRI_NONE)));
+            for (const char t : {'N', 'T'})
+                bytes = std::max(bytes, call_bytes(h, pl, tc_plan<T>(h, t, t, um, un, width,
+                                                                     gfip::TRI_NONE)));
         };
         // forward, the unknowns after each whole panel; backward, those before each panel
         for (int64_t p0 = 0; p0 < na; p0 += gfip::TRSM_PANEL) {

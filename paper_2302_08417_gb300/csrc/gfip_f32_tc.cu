@@ -25,24 +25,7 @@ using tc::KB;
 using tc::PLANE_BYTES;
 using tc::TM;
 
-constexpr uint32_t LOW_BITS = (127u - 100u) << 23;   // 2^-100
-constexpr uint32_t HIGH_BITS = (127u + 55u) << 23;   // 2^55
 constexpr int PITCH = TM + 1;
-
-// Two floats' planes as BF16 pairs (first element in the low half).
-__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &p1, uint32_t &p2,
-                                           uint32_t &p3)
-{
-    auto pack = [](float lo, float hi) -> uint32_t {
-        const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-        return *reinterpret_cast<const uint32_t *>(&v);
-    };
-    p1 = pack(x0, x1);
-    const float r0 = x0 - __uint_as_float(p1 << 16);
-    const float r1 = x1 - __uint_as_float(p1 & 0xFFFF0000u);
-    p2 = pack(r0, r1);
-    p3 = pack(r0 - __uint_as_float(p2 << 16), r1 - __uint_as_float(p2 & 0xFFFF0000u));
-}
 
 // Planes of one 128 x 32 block of an operand (one launch covers both).  The block is read
 // coalesced into shared memory; each thread then takes 8 consecutive k of one row and writes
@@ -81,8 +64,7 @@ __global__ void __launch_bounds__(256) split_kernel(F32SplitArgs a, F32SplitArgs
     for (int q = 0; q < PER; ++q) {
         const int r = a.contig_rows ? tid % TM : tid / KB + 8 * q;
         const int c = a.contig_rows ? tid / TM + 2 * q : tid % KB;
-        const uint32_t m = __float_as_uint(v[q]) & 0x7FFFFFFFu;
-        bad = bad || (m != 0u && m - LOW_BITS >= HIGH_BITS - LOW_BITS);
+        bad = bad || tc::outside_split(v[q]);
         tile[c * PITCH + r] = v[q];
     }
     if (__syncthreads_or(bad)) {
@@ -97,7 +79,7 @@ __global__ void __launch_bounds__(256) split_kernel(F32SplitArgs a, F32SplitArgs
         uint32_t p[3][4];
 #pragma unroll
         for (int h = 0; h < 4; ++h)
-            split_pair(src[2 * h * PITCH], src[(2 * h + 1) * PITCH], p[0][h], p[1][h], p[2][h]);
+            tc::split_pair(src[2 * h * PITCH], src[(2 * h + 1) * PITCH], p[0][h], p[1][h], p[2][h]);
 #pragma unroll
         for (int s = 0; s < 3; ++s)
             *reinterpret_cast<uint4 *>(dst + s * PLANE_BYTES + o * 16) =
@@ -106,6 +88,15 @@ __global__ void __launch_bounds__(256) split_kernel(F32SplitArgs a, F32SplitArgs
 }
 
 }  // namespace f32tc
+
+cudaError_t launch_f32_split(const F32SplitArgs &a, int k, int kt, unsigned int *gate,
+                             cudaStream_t s)
+{
+    F32SplitArgs none{};
+    f32tc::split_kernel<<<static_cast<unsigned int>((int64_t)a.row_blocks * kt), 256, 0, s>>>(
+        a, none, k, kt, nullptr, 0, gate);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_f32_tc(const TcParams &p, const F32SplitArgs &a, const F32SplitArgs &b, int k,
                           unsigned int *gate, int sms, cudaStream_t s)

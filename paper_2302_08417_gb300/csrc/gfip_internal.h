@@ -175,6 +175,31 @@ struct F32SplitArgs {
 cudaError_t launch_f32_tc(const TcParams &p, const F32SplitArgs &a, const F32SplitArgs &b, int k,
                           unsigned int *gate, int sms, cudaStream_t s);
 
+// Splits one operand only.
+cudaError_t launch_f32_split(const F32SplitArgs &a, int k, int kt, unsigned int *gate,
+                             cudaStream_t s);
+
+// Large FP32 products with at most 128 rows or columns (gfip_f32_skinny.cu): the large operand is
+// read where it lies, the small one from its planes.
+struct SkinnyParams {
+    const float *X;          // the large operand, element (row, p) at X[row + p*ld]
+    int64_t ld;
+    int rows, k;
+    const uint8_t *planes;   // the small operand's planes, one 128-row block
+    int n16;                 // its rows, rounded up to a multiple of 16
+    int kt, tiles;           // 32-wide k blocks; 128-row blocks of the large operand
+    int splits, units;       // k ranges; tiles * splits
+    float *partial;          // [splits][tiles][n16][128]
+    unsigned int *gate;      // set when an element is outside the range of the split
+    unsigned int *status;
+    unsigned long long wait_ns;
+};
+// Splits the small operand, runs the product and adds the k ranges into C (big_is_row: the large
+// operand's rows are C's rows), which is untouched when *gate is set.
+cudaError_t launch_f32_skinny(const SkinnyParams &p, const F32SplitArgs &small, float *C,
+                              int64_t ldc, int big_is_row, float alpha, float beta, int sms,
+                              cudaStream_t s);
+
 // FP64 GEMM emulated with BF16 digit products on the tensor cores (gfip_ozaki.cu).
 struct OzakiParams {
     const double *A;

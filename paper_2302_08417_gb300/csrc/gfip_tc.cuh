@@ -351,6 +351,32 @@ constexpr int F32_STAGES = 4;
 constexpr uint32_t F32_BYTES = F32_PLANES * PLANE_BYTES;
 static_assert(F32_STAGES * 2 * F32_PLANES <= SLOTS && F32_STAGES <= MAX_ASLOTS, "stages fit");
 
+// The range in which an FP32 element's split into three BF16 planes is exact and safe
+// (gfip_f32_tc.cu): zero, or a magnitude in [2^-100, 2^55).
+constexpr uint32_t LOW_BITS = (127u - 100u) << 23;   // 2^-100
+constexpr uint32_t HIGH_BITS = (127u + 55u) << 23;   // 2^55
+
+__device__ __forceinline__ bool outside_split(float x)
+{
+    const uint32_t m = __float_as_uint(x) & 0x7FFFFFFFu;
+    return m != 0u && m - LOW_BITS >= HIGH_BITS - LOW_BITS;
+}
+
+// Two floats' planes as BF16 pairs (first element in the low half).
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &p1, uint32_t &p2,
+                                           uint32_t &p3)
+{
+    auto pack = [](float lo, float hi) -> uint32_t {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+        return *reinterpret_cast<const uint32_t *>(&v);
+    };
+    p1 = pack(x0, x1);
+    const float r0 = x0 - __uint_as_float(p1 << 16);
+    const float r1 = x1 - __uint_as_float(p1 & 0xFFFF0000u);
+    p2 = pack(r0, r1);
+    p3 = pack(r0 - __uint_as_float(p2 << 16), r1 - __uint_as_float(p2 & 0xFFFF0000u));
+}
+
 // Digits: `na` A slots used round robin, then `nb` B stages of `planes` slots.
 struct Ring {
     int na, nb;

@@ -53,6 +53,27 @@ def test_fp32_shapes(runner, m, n, k):
     assert runner.h.status() == 0
 
 
+SKINNY = [("N", "T", 64, 8200, 1500), ("T", "T", 120, 9001, 1027), ("N", "N", 8200, 100, 1499),
+          ("N", "T", 9000, 128, 1090)]
+
+
+@pytest.mark.parametrize("ta,tb,m,n,k", SKINNY)
+def test_fp32_skinny(runner, ta, tb, m, n, k):
+    """At most 128 rows or columns: the large operand is split on its way to the MMA."""
+    p = inputs.problem(m + n + k, ta, tb, m, n, k, -0.75, 0.5, 7, 3, 5, dtype=np.float32)
+    got, guard = runner.run(p)
+    gu.assert_close(p, got)
+    gu.assert_gap_untouched(p, got, guard)
+    # an element outside the split's range in the large operand: the whole product is the FFMA
+    # kernel's, beta * C applied once
+    q = inputs.problem(m + n + k, ta, tb, m, n, k, 1.0, 0.5, 1, 1, 1, dtype=np.float32)
+    big, ld = (q.A, q.lda) if n <= m else (q.B, q.ldb)
+    big[40 + 900 * ld] = 1e25
+    got, _ = runner.run(q)
+    gu.assert_close(q, got)
+    assert runner.h.status() == 0
+
+
 @pytest.mark.parametrize("ea,eb", [(-99, 55), (-101, 30), (-115, 115), (-60, -60), (20, 56)])
 def test_fp32_magnitudes(runner, ea, eb):
     """Operands whose low planes are still normal BF16 numbers, and ones that would leave the
