@@ -30,7 +30,7 @@ constexpr int PITCH = TM + 1;
 // Planes of one 128 x 32 block of an operand (one launch covers both).  The block is read
 // coalesced into shared memory; each thread then takes 8 consecutive k of one row and writes
 // one 16-byte chunk per plane, consecutive threads consecutive chunks.  Bound by HBM: 4 bytes
-// read and 6 written per element.
+// read and 6 written per element (both operands of 4096^3: 335 MB in 63 us).
 __global__ void __launch_bounds__(256) split_kernel(F32SplitArgs a, F32SplitArgs b, int kdim,
                                                     int kblocks, unsigned int *counter,
                                                     int counters, unsigned int *gate)

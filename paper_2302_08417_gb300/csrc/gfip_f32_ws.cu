@@ -1,5 +1,6 @@
-// FP32 GEMM on the warp-specialised tile core (gfip_ws.cuh): the launch every dense FP32
-// GEMM of the library takes (fused, direct and pack-then-compute alike).
+// FP32 GEMM on the warp-specialised tile core (gfip_ws.cuh): the launch of the dense FP32 GEMMs
+// (fused, direct and pack-then-compute alike) that neither the small kernels (gfip_small.cu) nor
+// the tensor cores (gfip_f32_tc.cu) compute.
 #include "gfip_ws.cuh"
 
 namespace gfip {

@@ -137,7 +137,8 @@ __device__ __forceinline__ long long to_fixed(double x, int e)
 // field of X at w_s taken as a signed number, plus the bit below it.  So no digit waits for
 // another, and as 128 + i is the BF16 number with fraction i (i < 128), a pair of digits is
 // two field extractions and one exact BF16 subtraction of 160.  (The remainders formed one
-// after the other in 64-bit arithmetic took 190 us an operand at 4096 x 4096, seven digits.)
+// after the other in 64-bit arithmetic took 190 us an operand at 4096 x 4096, seven digits; this
+// takes 71, 0.34 GB of it HBM traffic.)
 struct SplitArgs {
     const double *X;
     int64_t ld;
