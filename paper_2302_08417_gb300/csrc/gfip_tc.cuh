@@ -312,9 +312,25 @@ struct Unit {
 __device__ __forceinline__ Unit unit_of(const TcParams &p, int u)
 {
     Unit x;
+    const int mask = p.tmask_a ? p.tmask_a : p.tmask_b;
+    if (mask) {
+        // A triangular operand leaves tiles of 1 to all of the k blocks (TRMM): the longest come
+        // first, and every other round of the grid runs backwards, so that a CTA with a
+        // long tile gets a short one next (2048 x 2048: 68 blocks on the busiest SM, 96 in
+        // band order).
+        const int grid = static_cast<int>(gridDim.x);
+        const int round = u / grid, at = u - round * grid;
+        if (round & 1) u = round * grid + min(grid, p.units - round * grid) - 1 - at;
+    }
     x.split = u / p.tiles;
     x.tile = u - x.split * p.tiles;
-    if (p.tri != TRI_NONE) {
+    if (mask) {
+        const int across = p.tmask_a ? p.nt : p.mt, along = p.tmask_a ? p.mt : p.nt;
+        const int rank = x.tile / across, other = x.tile - rank * across;
+        const int line = (mask & TMASK_KEEP_GE) ? along - 1 - rank : rank;
+        x.i = p.tmask_a ? line : other;
+        x.j = p.tmask_a ? other : line;
+    } else if (p.tri != TRI_NONE) {
         // row r of the lower triangle holds tiles r (r + 1) / 2 .. + r
         int r = static_cast<int>((sqrtf(8.f * static_cast<float>(x.tile) + 1.f) - 1.f) * 0.5f);
         while (r * (r + 1) / 2 > x.tile) --r;
@@ -333,9 +349,7 @@ __device__ __forceinline__ Unit unit_of(const TcParams &p, int u)
         x.j = in_band / rows;
     }
     int lo = 0, hi = p.kt;
-    // a triangular operand leaves only part of k to the tile (TRMM)
-    const int mask = p.tmask_a ? p.tmask_a : p.tmask_b;
-    if (mask) {
+    if (mask) {   // the k blocks that the tile's rows of the triangular operand keep
         const int x0 = (p.tmask_a ? x.i : x.j) * TM;
         const int strict = (mask & TMASK_STRICT) ? 1 : 0;
         if (mask & TMASK_KEEP_GE)
