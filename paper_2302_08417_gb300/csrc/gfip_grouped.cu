@@ -484,6 +484,33 @@ __device__ Counts block_exclusive(const Counts &v, Counts *wsum, Counts *total)
                   base.pelems + inc.pelems - v.pelems};
 }
 
+// The same for one integer.
+__device__ int block_exclusive(int v, int *wsum, int *total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto inclusive = [&](int x) {
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        return x;
+    };
+    const int inc = inclusive(v);
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+        const int w = wsum[lane], winc = inclusive(w);
+        wsum[lane] = winc - w;
+        if (lane == 31) wsum[32] = winc;
+    }
+    __syncthreads();
+    const int base = wsum[warp];
+    *total = wsum[32];
+    __syncthreads();
+    return base + inc - v;
+}
+
 // One CTA of 1024 threads turns the per-rank counts into the unit prefix sums the GEMM
 // kernel searches and gives each split problem its arrival counters and partial-sum space,
 // 1024 ranks at a time (coalesced loads, warp-shuffle scans).  With a plan, a split problem
@@ -493,6 +520,7 @@ __device__ Counts block_exclusive(const Counts &v, Counts *wsum, Counts *total)
 template <typename T> __global__ void __launch_bounds__(1024) scan_kernel(const GroupParams<T> gp)
 {
     __shared__ Counts wsum[33];
+    __shared__ int wunits[33];
     const int count = gp.count;
     const int tid = threadIdx.x;
     constexpr int KC = Pipe<T>::KC;
@@ -505,6 +533,20 @@ template <typename T> __global__ void __launch_bounds__(1024) scan_kernel(const 
         Counts v = next;
         if (r + 1024 < count)
             next = Counts{gp.units[r + 1024], gp.stiles[r + 1024], gp.pelems[r + 1024]};
+        // 1024 ranks without a split problem have only their units to scan (the usual plan: a
+        // third of the time of the two scans of three counts)
+        if (!__syncthreads_or(v.stiles > 0)) {
+            int tot;
+            const int before = block_exclusive(v.units, wunits, &tot) + carry.units;
+            carry.units += tot;
+            if (r < count) {
+                GroupDesc<T> &d = gp.desc[r];
+                d.ctr_off = carry.stiles;
+                d.part_off = carry.pelems;
+                gp.prefix[r] = before;
+            }
+            continue;
+        }
         if (gp.plan != nullptr) {
             Counts tot;
             const Counts before = block_exclusive(v, wsum, &tot) + req_carry;
