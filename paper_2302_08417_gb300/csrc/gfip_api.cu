@@ -276,17 +276,25 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
             t.splits = s;
         }
     }
-    // Estimated times, ns, fitted to one GB300: 2048^3 87 us, 64 x 8192 x 8192 205 (its planes' 10
-    // bytes an element dominate) and, split on the way, 112; 100 x 2000 x 2000 29 and 37.
+    // Estimated times, ns, fitted to one GB300: 640^3 18 us, 2048^3 87, 64 x 8192 x 8192 205 (its
+    // planes' 10 bytes an element dominate) and, split on the way, 112; 100 x 2000 x 2000 29
+    // and 37.
     const double planes = (double)m * k + (tri ? 0.0 : (double)n * k);
     const double part = tri ? 0.5 : 1.0;
-    t.ns = 12000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost;
-    // at most 128 rows or columns against an operand that is read along memory
+    t.ns = 9000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost;
+    // at most 128 rows or columns against an operand that is read along memory: k blocks on the
+    // busiest SM, and the launch that adds the k ranges
     if (tri == gfip::TRI_NONE && !masked && std::min(m, n) <= 128 &&
-        (n <= m ? is_notrans(transa) : !is_notrans(transb)) && 14000 + 700.0 * t.cost < t.ns) {
-        t.skinny = true;
-        t.n16 = static_cast<int>((std::min(m, n) + 15) / 16 * 16);
-        t.ns = 14000 + 700.0 * t.cost;
+        (n <= m ? is_notrans(transa) : !is_notrans(transb))) {
+        const int n16 = static_cast<int>((std::min(m, n) + 15) / 16 * 16);
+        const int64_t rounds = ((int64_t)t.tiles * t.splits + h->sms - 1) / h->sms;
+        const double ns = 17000 + (double)rounds * ((t.kt + t.splits - 1) / t.splits) *
+                                      (600 + 3.2 * n16) + 1000.0 * t.splits;
+        if (ns < t.ns) {
+            t.skinny = true;
+            t.n16 = n16;
+            t.ns = ns;
+        }
     }
     const size_t plane = 128 * 32 * 2;
     size_t d = 0;
@@ -316,8 +324,8 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
 // arithmetic (8192 x 8192 x 64: 7.19 ms against 7.27; 1500 x 1500 x 64: 272 us against 251).
 //
 // FP32: where the estimated time, in ns, is below the tensor cores' (or the FFMA core's, where
-// those cannot be used).  The estimates are fits on one GB300: 512^3 takes 14 us here and 24 on
-// the tensor cores, 640^3 24 on both, 2000 x 2000 x 16 33 here and 23 on either other path.
+// those cannot be used).  The estimates are fits on one GB300: 512^3 takes 14 us here and 17 on
+// the tensor cores, 640^3 24 and 18, 2000 x 2000 x 16 33 and 16 (23 on the FFMA core).
 template <typename T>
 bool use_small(const Handle *h, const TcPlan &tc, int64_t m, int64_t n, int64_t k, int tri)
 {

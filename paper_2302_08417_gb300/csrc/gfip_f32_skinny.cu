@@ -40,6 +40,8 @@ constexpr int THREADS = 64 + SPLIT_WARPS * 32;
 constexpr int PER = 8;             // its elements per thread and block
 static_assert(SPLIT_WARPS * 32 * PER == TM * KB, "a block");
 constexpr int CHUNK = tc::F32_CHUNK_BLOCKS;
+constexpr int LAG = CHUNK > 2 ? 2 : 1;   // blocks into the next chunk that one is drained
+static_assert(CHUNK > LAG, "a chunk is drained before the next one ends");
 static_assert(2 * PLANES * STAGES <= tc::SLOTS && STAGES <= tc::MAX_ASLOTS, "stages fit");
 
 struct Unit {
@@ -250,8 +252,8 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
             for (int d = 0; d < DEPTH; ++d) {
                 const int b = b0 + d;   // block within the unit
                 if (b >= len || !ok) break;
-                // a chunk is drained two blocks into the next, when its MMAs are through
-                if (b % CHUNK == 2) drain_to(b / CHUNK);
+                // a chunk is drained LAG blocks into the next, when its MMAs are through
+                if (b % CHUNK == LAG) drain_to(b / CHUNK);
                 if (!ok) break;
                 ok = tc::mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
                 if (!ok) break;

@@ -71,6 +71,12 @@ struct Panel {
     __device__ __forceinline__ int row(int q) const { return lower_t ? q : pw - 1 - q; }
 };
 
+// Panels of up to this many blocks are staged by every CTA itself: their triangle is a few
+// loads a thread, less than the packing launch (64 unknowns and sides with the caller's copy of
+// B: 12.1 us a call; 16.4 from 100 unknowns on, with it), and both column buffers hold all
+// there is.
+constexpr int SELF_BLOCKS = 3;
+
 // Packs the panel: CTA (bi, bj), bi >= bj, writes the 32 x 32 block of rows 32 bi, columns 32 bj.
 __global__ void __launch_bounds__(256) pack_kernel(const Panel p, int nb, float *image)
 {
@@ -257,6 +263,33 @@ __device__ __forceinline__ void move_sides(const Panel &p, float *B, int64_t vst
 }
 static_assert(NV == 2 * WARPS, "two sides a warp");
 
+// The whole triangle of a panel of at most SELF_BLOCKS blocks, straight into the images.
+__device__ __forceinline__ void stage_self(const Panel &p, int nb, Smem &sm)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int bi = 0; bi < nb; ++bi)
+        for (int bj = 0; bj <= bi; ++bj) {
+            float *dst = bi == bj ? sm.head + 2 * BLK * nb + bi * BLK * BLK
+                                  : sm.col[bj] + (bi - bj - 1) * BLK;
+            const int pitch = bi == bj ? BLK : below(nb, bj);
+#pragma unroll
+            for (int c = 0; c < BLK / WARPS; ++c) {
+                const int a = w + WARPS * c;   // lanes along the contiguous direction of A
+                const int i = p.along_q ? lane : a, j = p.along_q ? a : lane;
+                const int q = bi * BLK + i, d = bj * BLK + j;
+                dst[j * pitch + i] =
+                    q > d && q < p.pw ? p.A0[(int64_t)q * p.sq + (int64_t)d * p.sd] : 0.f;
+            }
+        }
+    const int q = threadIdx.x;
+    if (q < nb * BLK) {
+        const float t = !p.unit && q < p.pw ? p.A0[(int64_t)q * (p.sq + p.sd)] : 1.f;
+        sm.head[q] = t;
+        sm.head[nb * BLK + q] = 1.f / t;
+    }
+}
+static_assert(SELF_BLOCKS <= 3 && SELF_BLOCKS * BLK <= WARPS * 32, "two column buffers, one pass");
+
 __global__ void __launch_bounds__(WARPS * 32, 1)
     panel_kernel(float *B, int64_t vstride, int64_t estride, int nvec, const Panel p,
                  const float *image, unsigned int *status)
@@ -265,8 +298,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5;
     const int nb = (p.pw + BLK - 1) / BLK;
+    const bool self = image == nullptr;
     auto fetch_columns = [&](int bk) {   // block bk's columns below it, if there are any
-        if (bk + 1 < nb)
+        if (bk + 1 < nb && !self)
             fetch(sm.col[bk & 1], image + columns_at(nb, bk), BLK * below(nb, bk),
                   &sm.full[bk & 1]);
     };
@@ -275,13 +309,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&sm.full[i]))
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fetch(sm.head, image, head_floats(nb), &sm.full[2]);
+        if (!self) fetch(sm.head, image, head_floats(nb), &sm.full[2]);
         fetch_columns(0);
         fetch_columns(1);
     }
+    if (self) stage_self(p, nb, sm);
     move_sides<false>(p, B, vstride, estride, nvec, nb * BLK, sm);
     __syncthreads();
-    bool ok = arrived(&sm.full[2], 0);
+    bool ok = self || arrived(&sm.full[2], 0);
     if (warp == 0 && ok) solve_block(sm, nb, 0);
     ok = __syncthreads_and(ok);
     int bk = 0;
@@ -293,7 +328,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
             const float v = -x[j * XP];
             nx[j] = make_float2(v, v);
         }
-        ok = arrived(&sm.full[bk & 1], (bk >> 1) & 1);
+        ok = self || arrived(&sm.full[bk & 1], (bk >> 1) & 1);
         const int units = (nb - 1 - bk) * (BLK / 16);
         if (warp < 2) {
             update_rows(sm, nb, bk, warp, nx);   // the next block's rows
@@ -356,7 +391,10 @@ cudaError_t launch_trsm_panel_f32(float *B, int64_t vstride, int64_t estride, in
     p.unit = unit;
     p.pw = pw;
     const int nb = (pw + BLK - 1) / BLK;
-    pack_kernel<<<nb * (nb + 1) / 2, 256, 0, s>>>(p, nb, image);
+    if (nb <= SELF_BLOCKS)
+        image = nullptr;
+    else
+        pack_kernel<<<nb * (nb + 1) / 2, 256, 0, s>>>(p, nb, image);
     panel_kernel<<<(nvec + NV - 1) / NV, WARPS * 32, sizeof(Smem), s>>>(B, vstride, estride, nvec,
                                                                         p, image, status);
     return cudaGetLastError();
