@@ -411,6 +411,12 @@ int gemm_entry(gfip_handle_t handle, Variant v, char transa, char transb, int64_
 cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<float> &p,
                       unsigned char *data)
 {
+    // k blocks (of 32) per accumulation on the tensor cores, whose truncation shows as a bias that
+    // grows with a chunk's length (entries in [0, 1], relative error: 8e-8 with 64 k, 1.5e-7 with
+    // 128, 3.1e-7 with 256), while the FFMA chain's error grows with k (8e-8 to 1.2e-7 at 64 to
+    // 700, 8e-7 at 4096).  Short chunks cost drains: 4096^3 takes 602 us with 64, 540 with 128, 505
+    // with 256.
+    const int chunk = p.k <= 1024 ? 2 : 4;
     if (t.skinny) {
         const bool big_is_row = p.n <= p.m;   // op(A) is the large operand
         gfip::SkinnyParams q{};
@@ -424,6 +430,7 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
         q.tiles = t.tiles;
         q.splits = t.splits;
         q.units = t.tiles * t.splits;
+        q.chunk = chunk;
         q.partial = reinterpret_cast<float *>(data + t.off_partial);
         q.gate = p.gate;
         q.status = p.status;
@@ -457,6 +464,7 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
     q.tmask_b = p.tmask_b;
     q.splits = t.splits;
     q.units = t.tiles * t.splits;
+    q.chunk = chunk;
     q.partial = reinterpret_cast<float *>(data + t.off_partial);
     q.counter = reinterpret_cast<unsigned int *>(data + t.off_counter);
     q.gate = p.gate;

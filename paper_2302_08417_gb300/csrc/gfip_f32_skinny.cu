@@ -39,9 +39,6 @@ constexpr int SPLIT_WARPS = 16;
 constexpr int THREADS = 64 + SPLIT_WARPS * 32;
 constexpr int PER = 8;             // its elements per thread and block
 static_assert(SPLIT_WARPS * 32 * PER == TM * KB, "a block");
-constexpr int CHUNK = tc::F32_CHUNK_BLOCKS;
-constexpr int LAG = CHUNK > 2 ? 2 : 1;   // blocks into the next chunk that one is drained
-static_assert(CHUNK > LAG, "a chunk is drained before the next one ends");
 static_assert(2 * PLANES * STAGES <= tc::SLOTS && STAGES <= tc::MAX_ASLOTS, "stages fit");
 
 struct Unit {
@@ -117,8 +114,8 @@ __device__ void issuer(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
     const uint32_t base = tc::desc_low(tc::saddr(sm.plane[0]));
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit x = unit_of(p, u);
-        for (int k0 = x.kb0; k0 < x.kb1 && ok; k0 += CHUNK, ++chunks) {
-            const int k1 = min(x.kb1, k0 + CHUNK);
+        for (int k0 = x.kb0; k0 < x.kb1 && ok; k0 += p.chunk, ++chunks) {
+            const int k1 = min(x.kb1, k0 + p.chunk);
             const uint32_t buf = chunks & 1u;
             ok = tc::mbar_wait(&sm.tempty[buf], ((chunks >> 1) & 1u) ^ 1u, sm, p.status,
                                p.wait_ns);
@@ -199,6 +196,7 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
     const int quarter = warp & 3, part = (warp - 2) >> 2;   // tensor-memory lanes and columns
     const int cols = p.n16 / 4;              // accumulator columns of this part
     const Block mine(t);
+    const int lag = p.chunk > 2 ? 2 : 1;
     int stage = 0;
     uint32_t lap = 0;
     uint32_t drained = 0;                    // chunks drained, over all units
@@ -252,8 +250,8 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
             for (int d = 0; d < DEPTH; ++d) {
                 const int b = b0 + d;   // block within the unit
                 if (b >= len || !ok) break;
-                // a chunk is drained LAG blocks into the next, when its MMAs are through
-                if (b % CHUNK == LAG) drain_to(b / CHUNK);
+                // a chunk is drained a block or two into the next, when its MMAs are through
+                if ((b & (p.chunk - 1)) == lag) drain_to(b / p.chunk);
                 if (!ok) break;
                 ok = tc::mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
                 if (!ok) break;
@@ -271,7 +269,7 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
                 left -= KB;
             }
         }
-        if (ok) drain_to((len + CHUNK - 1) / CHUNK);
+        if (ok) drain_to((len + p.chunk - 1) / p.chunk);
         if (!ok) break;
         // partial sums of the unit: [small row][128 rows of the large operand]
         float *out = p.partial + ((int64_t)u * p.n16 + part * cols) * TM + quarter * 32 + lane;

@@ -4,9 +4,9 @@
 // nearest leaves a remainder of at most 2^-9 of what it rounded, and 24 significant bits fit
 // three planes of 8.  The tile core (gfip_tc.cuh) forms a1 b1 + (a1 b2 + a2 b1 + a1 b3 + a2 b2 +
 // a3 b1); the products left out are below 2^-25 of |a b|.  a1 b1 and the smaller products are
-// accumulated apart, for 256 k at a time, and the chunks are added in FP32 with rounding to
-// nearest, which keeps the sum more exact than one chain of k FP32 multiply-adds (the
-// FFMA cores' order).  Packing is where the split happens: one pass reads the strided
+// accumulated apart, for 64 or 128 k at a time (launch_tc in gfip_api.cu), and the chunks are
+// added in FP32 with rounding to nearest, which keeps the sum at least as exact as one chain of k
+// FP32 multiply-adds (the FFMA cores' order), also where all terms have one sign.  Packing is where the split happens: one pass reads the strided
 // operands (masking triangular ones) and writes the plane tiles the MMA reads.
 //
 // The split is exact while no plane leaves BF16's normal range and no product or sum FP32's:

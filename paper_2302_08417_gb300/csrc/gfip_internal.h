@@ -150,6 +150,7 @@ struct TcParams {
     int tri;             // TRI_*: the triangle of C computed (SYRK)
     int tmask_a, tmask_b;  // triangular operand (TRMM): which k a tile needs, see TriMask
     int splits;          // k-ranges per tile (FP32), added by the last to finish
+    int chunk;           // FP32: k blocks per accumulation on the tensor cores
     int units;           // tiles * splits
     const int *ea, *eb;  // digits: row exponents of op(A), column exponents of op(B)
     float *partial;      // [tiles][splits] partial tiles of 128 x 128 (splits > 1)
@@ -189,6 +190,7 @@ struct SkinnyParams {
     int n16;                 // its rows, rounded up to a multiple of 16
     int kt, tiles;           // 32-wide k blocks; 128-row blocks of the large operand
     int splits, units;       // k ranges; tiles * splits
+    int chunk;               // k blocks per accumulation on the tensor cores (a power of two)
     float *partial;          // [splits][tiles][n16][128]
     unsigned int *gate;      // set when an element is outside the range of the split
     unsigned int *status;

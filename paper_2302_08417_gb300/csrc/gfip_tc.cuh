@@ -20,7 +20,7 @@
 // MMA of N = 256: it reads 12 KB of operands per 128 clocks where two of N = 128 read 16 KB.
 //
 // Measured on one GB300: 4096^3 with 7 digits 4710 -> 2416 us (tensor pipe 75 % busy), 8192^3 38 ->
-// 63 TFLOP/s FP64-equivalent; FP32 4096^3 2513 us on the FFMA core -> 520 (265 TFLOP/s).
+// 63 TFLOP/s FP64-equivalent; FP32 4096^3 2513 us on the FFMA core -> 540 (254 TFLOP/s).
 //
 // Roles (one CTA per SM, 10 warps, persistent over the units of work):
 //   warp 0      producer.  Digits: per k block one bulk copy of the B planes the group needs (two
@@ -63,12 +63,6 @@ constexpr int EPI_WARPS = 8;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int DIGIT_BITS = 6;
 constexpr int EXACT_TERMS = 16384;       // digit products whose sum FP32 holds exactly
-// k per FP32 accumulation on the tensor cores before the sum moves to registers, where it is
-// added with rounding to nearest: short, because the tensor cores' accumulation truncates.
-#ifndef GFIP_F32_TC_CHUNK
-#define GFIP_F32_TC_CHUNK 256
-#endif
-constexpr int F32_CHUNK_BLOCKS = GFIP_F32_TC_CHUNK / KB;
 constexpr long long WAIT_POLLS = 1ll << 32;          // backstop, should the timer stall
 
 enum Kind : int { KIND_DIGITS_INT = 0, KIND_DIGITS_F64 = 1, KIND_F32 = 2 };
@@ -574,8 +568,8 @@ __device__ __forceinline__ void f32_issuer(const TcParams &p, Smem &sm, uint32_t
     const uint32_t base = desc_low(saddr(sm.plane[0]));
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit x = unit_of(p, u);
-        for (int k0 = x.kb0; k0 < x.kb1 && ok; k0 += F32_CHUNK_BLOCKS, ++chunks) {
-            const int k1 = min(x.kb1, k0 + F32_CHUNK_BLOCKS);
+        for (int k0 = x.kb0; k0 < x.kb1 && ok; k0 += p.chunk, ++chunks) {
+            const int k1 = min(x.kb1, k0 + p.chunk);
             const uint32_t buf = chunks & 1u;
             ok = mbar_wait(&sm.tempty[buf], ((chunks >> 1) & 1u) ^ 1u, sm, p.status, p.wait_ns);
             if (!ok) break;
@@ -707,7 +701,7 @@ template <int KIND> __device__ void epilogue(const TcParams &p, Smem &sm, uint32
         for (int c = 0; c < 64; ++c) acc[c] = Acc(0);
         for (int g = 0; g < groups; ++g) {
             const Group q =
-                KIND == KIND_F32 ? Group{2, 4, F32_CHUNK_BLOCKS} : group_of(g, p.planes);
+                KIND == KIND_F32 ? Group{2, 4, p.chunk} : group_of(g, p.planes);
             for (int k0 = x.kb0; k0 < x.kb1; k0 += q.chunk, ++chunks) {
                 const int buf = chunks % NBUF;
                 if (!mbar_wait(&sm.tfull[buf], (chunks / NBUF) & 1u, sm, p.status, p.wait_ns))

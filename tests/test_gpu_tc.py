@@ -40,6 +40,7 @@ def test_digit_counts_and_chunk_edges(runner, slices):
 
 
 @pytest.mark.parametrize("m,n,k", [(700, 650, 600), (2000, 1500, 16), (1030, 1100, 289),
+                                   (900, 700, 1024), (900, 700, 1025),
                                    (130, 8000, 255), (2100, 129, 1025), (300, 290, 7001)])
 def test_fp32_shapes(runner, m, n, k):
     for ta, tb in (("N", "N"), ("T", "T")):
