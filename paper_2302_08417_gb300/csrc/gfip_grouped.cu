@@ -531,8 +531,9 @@ template <typename T> __global__ void __launch_bounds__(1024) scan_kernel(const 
     for (int base = 0; base < count; base += 1024) {
         const int r = base + tid;
         Counts v = next;
-        if (r + 1024 < count)
-            next = Counts{gp.units[r + 1024], gp.stiles[r + 1024], gp.pelems[r + 1024]};
+        next = r + 1024 < count   // nothing past the last rank
+                   ? Counts{gp.units[r + 1024], gp.stiles[r + 1024], gp.pelems[r + 1024]}
+                   : Counts{0, 0, 0};
         // 1024 ranks without a split problem have only their units to scan (the usual plan: a
         // third of the time of the two scans of three counts)
         if (!__syncthreads_or(v.stiles > 0)) {

@@ -143,6 +143,42 @@ def test_full_batched_workload_matches_oracle(dev, dtype):
 
 
 @pytest.mark.parametrize("dtype", [np.float64, np.float32], ids=["f64", "f32"])
+@pytest.mark.parametrize("splits", [1, 2])
+@pytest.mark.parametrize("count", [1024, 1025, 1500, 2047, 3000])
+def test_counts_around_the_scan_width(dev, dtype, count, splits):
+    """Counts that end inside a scan of 1024 ranks: no rank past the last is counted, so the last
+    rank (in order of the batch: an invalid problem here) has no work but its own, split or not."""
+    probs = make_problems(count + splits, count, dtype, lo=4, hi=24)
+    batch, bufs = build_batch(probs, dev)
+    skipped = 0 if splits > 1 else count - 1
+    batch.ldc[skipped] = 0
+    if splits > 1:
+        plan = gr.Plan.uniform(batch, g.GFIP_GROUP_TILE_16X8, splits)
+        plan.order = torch.arange(count - 1, -1, -1, dtype=torch.int32, device=dev)
+        gr.run(batch, plan)
+    else:
+        gr.run(batch, g.GFIP_GROUP_TILE_TINY)
+    torch.cuda.synchronize()
+    flat = [b.cpu().numpy() for b in bufs]
+    assert np.array_equal(flat[skipped].view(np.uint8), probs[skipped].C0.view(np.uint8))
+    for q, (p, got) in enumerate(zip(probs, flat)):
+        if q != skipped:
+            gu.assert_close(p, got, label=f"problem {q} of {count}")
+    assert g.default_handle().status() == g.GFIP_STATUS_BAD_PROBLEM
+    # the last rank a valid, split or unsplit problem
+    batch, bufs = build_batch(probs, dev)
+    if splits > 1:
+        plan.order = torch.arange(count, dtype=torch.int32, device=dev)
+        gr.run(batch, plan)
+    else:
+        gr.run(batch, g.GFIP_GROUP_TILE_TINY)
+    torch.cuda.synchronize()
+    for q, (p, buf) in enumerate(zip(probs, bufs)):
+        gu.assert_close(p, buf.cpu().numpy(), label=f"problem {q} of {count}")
+    assert g.default_handle().status() == 0
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32], ids=["f64", "f32"])
 def test_graph_replay_and_autotune(dev, dtype):
     probs = make_problems(5, 200, dtype)
     batch, bufs = build_batch(probs, dev)
