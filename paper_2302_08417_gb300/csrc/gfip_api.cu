@@ -834,6 +834,27 @@ int trmm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     return GFIP_OK;
 }
 
+// Control words of a TRSM: those its updates' plans need, and, where an FP32 panel is packed, the
+// header at least (its packed triangle lies behind the control region).  0: a single panel that
+// runs without any, so that it needs no clearing.
+template <typename T> size_t trsm_ctrl(Handle *h, char side, bool lower_t, int64_t m, int64_t n)
+{
+    const bool left = side == 'L' || side == 'l';
+    const int na = (int)(left ? m : n), panel = gfip::TRSM_PANEL;
+    const int npanels = (na + panel - 1) / panel;
+    size_t ctrl = sizeof(T) == 4 && gfip::trsm_packs(std::min(panel, na)) ? kCtrlGranule : 0;
+    // A plan's control words grow with each dimension: the first update has the most unknowns
+    // left, and the second, where the last panel is a short one and comes first, the most terms.
+    for (int ps = 0; ps < std::min(2, npanels - 1); ++ps) {
+        const int p0 = (lower_t ? ps : npanels - 1 - ps) * panel, pw = std::min(panel, na - p0);
+        const int rest = lower_t ? na - p0 - pw : p0;
+        const Plan<T> pl = make_plan<T>(h, Variant::Fused, left ? rest : (int)m,
+                                        left ? (int)n : rest, pw);
+        ctrl = std::max(ctrl, round_up(pl.ctrl_needed, kCtrlGranule));
+    }
+    return ctrl;
+}
+
 // Workspace every panel update of a TRSM can run in (the FFMA or DFMA path's).
 template <typename T>
 size_t trsm_workspace_min(Handle *h, char side, int64_t m, int64_t n)
@@ -843,10 +864,11 @@ size_t trsm_workspace_min(Handle *h, char side, int64_t m, int64_t n)
     const bool left = side == 'L' || side == 'l';
     const int na = (int)(left ? m : n);
     const int pw = std::min(gfip::TRSM_PANEL, na);
-    const Plan<T> panel = make_plan<T>(h, Variant::Fused, (int)m, (int)n, pw);
-    // (a panel's packed triangle, FP32, is smaller than the plan's partial tiles or panels)
-    return std::max(total_bytes(h, panel),
-                    h->ctrl_bytes + (sizeof(T) == 4 ? gfip::trsm_image_bytes(pw) : 0));
+    Plan<T> panel = make_plan<T>(h, Variant::Fused, (int)m, (int)n, pw);
+    // a panel's packed triangle, FP32, lies where the update's partial tiles and panels do
+    if (sizeof(T) == 4)
+        panel.data_bytes = std::max(panel.data_bytes, gfip::trsm_image_bytes(pw));
+    return total_bytes(h, panel);
 }
 
 // ... and with room for the tensor-core path of the updates that take it.
@@ -900,13 +922,6 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
         if (h->ws == nullptr) return GFIP_ERR_WORKSPACE;
         if (trsm_workspace_min<T>(h, side, m, n) > h->ws_bytes) return GFIP_ERR_WORKSPACE;
     }
-    if (alpha != T(1)) {   // B := alpha B (alpha == 0: zeros, B not read)
-        if (gfip::launch_scale<T>(B, ldb, (int)m, (int)n, alpha, gfip::TRI_NONE, h->stream) !=
-            cudaSuccess)
-            return GFIP_ERR_CUDA;
-        if (alpha == T(0)) return GFIP_OK;
-    }
-    if (A == nullptr) return GFIP_ERR_NULLPTR;
     const bool left = side == 'L' || side == 'l';
     const bool trans = !is_notrans(transa);
     const bool lower_op = (uplo == 'L' || uplo == 'l') != trans;
@@ -914,6 +929,24 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     const bool unit = diag == 'U' || diag == 'u';
     const int na = (int)(left ? m : n);
     const char ta = trans ? 'T' : 'N';
+    unsigned char *image = nullptr;   // FP32: where a panel's triangle is packed
+    if (alpha != T(0)) {
+        // The control words are cleared before the first launch, for all panels.  While the
+        // stream is capturing they cannot be; a single packed panel, which needs no control
+        // word, is then solved without them: its triangle lies behind the region a first call
+        // would clear, and it reports no status, so it is staged without waits.
+        const size_t ctrl = trsm_ctrl<T>(h, side, lower_t, m, n);
+        image = h->ws + std::max(h->ctrl_bytes, ctrl);
+        if (const int rc = grow_ctrl(h, ctrl);
+            rc != GFIP_OK && !(rc == GFIP_ERR_CAPTURE && na <= gfip::TRSM_PANEL))
+            return rc;
+    }
+    if (alpha != T(1)) {   // B := alpha B (alpha == 0: zeros, B not read)
+        if (gfip::launch_scale<T>(B, ldb, (int)m, (int)n, alpha, gfip::TRI_NONE, h->stream) !=
+            cudaSuccess)
+            return GFIP_ERR_CUDA;
+        if (alpha == T(0)) return GFIP_OK;
+    }
     // B[rest] -= op(A)[rest, k0:k0+kb] X[k0:k0+kb] for the unknowns r0..r1-1 (side L), or
     // B[:, rest] -= X[:, k0:k0+kb] op(A)[k0:k0+kb, rest] (side R)
     auto update = [&](int k0, int kb, int r0, int r1) -> int {
@@ -940,10 +973,10 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
         cudaError_t e;
         if constexpr (sizeof(T) == 4) {
             // the packed triangle takes the bytes the update's GEMM uses afterwards
-            e = gfip::launch_trsm_panel_f32(Bp, vstride, estride, nvec, A, lda, trans, p0, pw,
-                                            lower_t, left ? 0 : 1, unit,
-                                            reinterpret_cast<float *>(h->ws + h->ctrl_bytes),
-                                            reinterpret_cast<unsigned int *>(h->ws), h->stream);
+            e = gfip::launch_trsm_panel_f32(
+                Bp, vstride, estride, nvec, A, lda, trans, p0, pw, lower_t, left ? 0 : 1, unit,
+                reinterpret_cast<float *>(image),
+                h->ctrl_bytes > 0 ? reinterpret_cast<unsigned int *>(h->ws) : nullptr, h->stream);
         } else {
             e = gfip::launch_trsm_panel_f64(Bp, vstride, estride, nvec, A, lda, trans, p0, pw,
                                             lower_t, left ? 0 : 1, unit, h->stream);

@@ -227,7 +227,8 @@ cudaError_t launch_ozaki(const OzakiParams &p, int sms, cudaStream_t s);
 // Triangular solve: one launch solves a panel of at most TRSM_PANEL unknowns (op(A)'s diagonal
 // block at (k0, k0), transposed for side 'R') for every right-hand side; vector v's element i is
 // B[v*vstride + i*estride].  FP64 in gfip_trsm.cu; FP32 in gfip_trsm_f32.cu, which packs the
-// panel's triangle into `image` (trsm_image_bytes(), 16-byte aligned) first.
+// panel's triangle into `image` (trsm_image_bytes(), 16-byte aligned) first when trsm_packs().
+// status: null when there is no cleared status word; the panel is then staged without waits.
 constexpr int TRSM_PANEL = 512;
 cudaError_t launch_trsm_panel_f64(double *B, int64_t vstride, int64_t estride, int nvec,
                                   const double *A, int64_t lda, int a_trans, int k0, int pw,
@@ -237,6 +238,7 @@ cudaError_t launch_trsm_panel_f32(float *B, int64_t vstride, int64_t estride, in
                                   int lower_t, int transpose_t, int unit, float *image,
                                   unsigned int *status, cudaStream_t s);
 size_t trsm_image_bytes(int pw);
+bool trsm_packs(int pw);
 
 // Grouped GEMM (gfip_grouped.cu): many independent problems in one persistent launch, each
 // problem with its own warp-tile shape and k-split factor.

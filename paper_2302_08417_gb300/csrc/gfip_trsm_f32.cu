@@ -299,24 +299,40 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     const int tid = threadIdx.x, warp = tid >> 5;
     const int nb = (p.pw + BLK - 1) / BLK;
     const bool self = image == nullptr;
+    const bool plain = !self && status == nullptr;   // staged by the threads: nothing to wait for
     auto fetch_columns = [&](int bk) {   // block bk's columns below it, if there are any
-        if (bk + 1 < nb && !self)
+        if (bk + 1 < nb)
             fetch(sm.col[bk & 1], image + columns_at(nb, bk), BLK * below(nb, bk),
                   &sm.full[bk & 1]);
+    };
+    auto copy = [&](float *dst, const float *src, int n) {
+        for (int i = 4 * tid; i < n; i += 4 * WARPS * 32)
+            *reinterpret_cast<float4 *>(dst + i) = *reinterpret_cast<const float4 *>(src + i);
+    };
+    auto copy_columns = [&](int bk) {
+        if (bk + 1 < nb) copy(sm.col[bk & 1], image + columns_at(nb, bk), BLK * below(nb, bk));
     };
     if (tid == 0) {
         for (int i = 0; i < 3; ++i)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&sm.full[i]))
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (!self) fetch(sm.head, image, head_floats(nb), &sm.full[2]);
-        fetch_columns(0);
-        fetch_columns(1);
+        if (!self && !plain) {
+            fetch(sm.head, image, head_floats(nb), &sm.full[2]);
+            fetch_columns(0);
+            fetch_columns(1);
+        }
     }
     if (self) stage_self(p, nb, sm);
+    if (plain) {
+        copy(sm.head, image, head_floats(nb));
+        copy_columns(0);
+        copy_columns(1);
+    }
     move_sides<false>(p, B, vstride, estride, nvec, nb * BLK, sm);
     __syncthreads();
-    bool ok = self || arrived(&sm.full[2], 0);
+    const bool staged = self || plain;
+    bool ok = staged || arrived(&sm.full[2], 0);
     if (warp == 0 && ok) solve_block(sm, nb, 0);
     ok = __syncthreads_and(ok);
     int bk = 0;
@@ -328,7 +344,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
             const float v = -x[j * XP];
             nx[j] = make_float2(v, v);
         }
-        ok = self || arrived(&sm.full[bk & 1], (bk >> 1) & 1);
+        ok = staged || arrived(&sm.full[bk & 1], (bk >> 1) & 1);
         const int units = (nb - 1 - bk) * (BLK / 16);
         if (warp < 2) {
             update_rows(sm, nb, bk, warp, nx);   // the next block's rows
@@ -340,7 +356,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
             for (int u = 1 + warp; u < units; u += WARPS - 1) update_rows(sm, nb, bk, u, nx);
         }
         ok = __syncthreads_and(ok);
-        if (tid == 0 && ok) fetch_columns(bk + 2);   // into the buffer just read
+        // into the buffer just read
+        if (plain)
+            copy_columns(bk + 2);
+        else if (tid == 0 && ok && !self)
+            fetch_columns(bk + 2);
     }
     if (!ok) {
         // a copy never arrived: leave B as it is, and no copy behind (fetched, not awaited yet)
@@ -354,6 +374,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
 }
 
 }  // namespace trsm32
+
+bool trsm_packs(int pw)
+{
+    return pw > trsm32::SELF_BLOCKS * trsm32::BLK;
+}
 
 size_t trsm_image_bytes(int pw)
 {
@@ -391,7 +416,7 @@ cudaError_t launch_trsm_panel_f32(float *B, int64_t vstride, int64_t estride, in
     p.unit = unit;
     p.pw = pw;
     const int nb = (pw + BLK - 1) / BLK;
-    if (nb <= SELF_BLOCKS)
+    if (!trsm_packs(pw))
         image = nullptr;
     else
         pack_kernel<<<nb * (nb + 1) / 2, 256, 0, s>>>(p, nb, image);
