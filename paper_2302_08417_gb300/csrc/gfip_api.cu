@@ -32,6 +32,7 @@ constexpr int kMinSplitRun = 8;              // shortest k run per CTA in a spli
 // k-blocks, so a 128 x 128 tile is summed from a few partial tiles, not from one per k-block.
 constexpr int kMinSplitRunF32 = 4;
 constexpr unsigned long long kOzakiWaitNs = 2000000000ull;  // 2 s per pipeline wait
+constexpr unsigned long long kF32WaitNs = 2000000000ull;
 // FP32 products of at least this many terms may run on the tensor cores (gfip_f32_tc.cu): with
 // fewer, the terms the split leaves out would show beside the rounding of the sum.
 constexpr int64_t kTcMinK = 16;
@@ -51,6 +52,8 @@ struct Handle {
     int packer = GFIP_PACKER_AUTO;
     unsigned long long oz_wait_ns = kOzakiWaitNs;  // budget of the emulation kernel's waits
     int oz_inject = 0;                             // test hook (gfip_debug_ozaki_timeout)
+    unsigned long long f32_wait_ns = kF32WaitNs;   // budget of the FP32 kernels' waits
+    int f32_inject = 0;                            // test hook (gfip_debug_f32_timeout)
     int last_launches = 0;
     int last_grid = 0;
     int bps_f64 = 0;
@@ -434,7 +437,8 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
         q.partial = reinterpret_cast<float *>(data + t.off_partial);
         q.gate = p.gate;
         q.status = p.status;
-        q.wait_ns = kOzakiWaitNs;
+        q.wait_ns = p.wait_ns;
+        q.inject_timeout = p.inject_timeout;
         const gfip::F32SplitArgs small{big_is_row ? p.B : p.A,
                                        big_is_row ? p.ldb : p.lda,
                                        big_is_row ? p.n : p.m,
@@ -469,7 +473,8 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
     q.counter = reinterpret_cast<unsigned int *>(data + t.off_counter);
     q.gate = p.gate;
     q.status = p.status;
-    q.wait_ns = kOzakiWaitNs;
+    q.wait_ns = p.wait_ns;
+    q.inject_timeout = p.inject_timeout;
     const gfip::F32SplitArgs a{p.A, p.lda, p.m, p.a_contig_m, t.mt, p.tmask_a, data + t.off_a};
     gfip::F32SplitArgs b{p.B, p.ldb, p.n, p.b_contig_n, t.nt, p.tmask_b, data + t.off_b};
     if (p.tri != gfip::TRI_NONE) b.row_blocks = 0;   // both roles read the planes of A
@@ -561,6 +566,8 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
     p.done_count = reinterpret_cast<unsigned int *>(h->ws + kDoneCountOffset);
     p.pack_count = reinterpret_cast<unsigned long long *>(h->ws + kPackCountOffset);
     p.tile_next = reinterpret_cast<unsigned long long *>(h->ws + kTileNextOffset);
+    p.wait_ns = h->f32_wait_ns;
+    p.inject_timeout = h->f32_inject;
 
     int launches = 0;
     if constexpr (sizeof(T) == 4) {
@@ -976,7 +983,8 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
             e = gfip::launch_trsm_panel_f32(
                 Bp, vstride, estride, nvec, A, lda, trans, p0, pw, lower_t, left ? 0 : 1, unit,
                 reinterpret_cast<float *>(image),
-                h->ctrl_bytes > 0 ? reinterpret_cast<unsigned int *>(h->ws) : nullptr, h->stream);
+                h->ctrl_bytes > 0 ? reinterpret_cast<unsigned int *>(h->ws) : nullptr,
+                h->f32_wait_ns, h->f32_inject, h->stream);
         } else {
             e = gfip::launch_trsm_panel_f64(Bp, vstride, estride, nvec, A, lda, trans, p0, pw,
                                             lower_t, left ? 0 : 1, unit, h->stream);
@@ -1072,6 +1080,15 @@ int gfip_debug_ozaki_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns)
     if (h == nullptr) return GFIP_ERR_HANDLE;
     h->oz_inject = enable ? 1 : 0;
     h->oz_wait_ns = wait_ns ? wait_ns : kOzakiWaitNs;
+    return GFIP_OK;
+}
+
+int gfip_debug_f32_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns)
+{
+    Handle *h = get(handle);
+    if (h == nullptr) return GFIP_ERR_HANDLE;
+    h->f32_inject = enable ? 1 : 0;
+    h->f32_wait_ns = wait_ns ? wait_ns : kF32WaitNs;
     return GFIP_OK;
 }
 

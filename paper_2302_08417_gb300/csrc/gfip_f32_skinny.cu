@@ -39,7 +39,7 @@ constexpr int SPLIT_WARPS = 16;
 constexpr int THREADS = 64 + SPLIT_WARPS * 32;
 constexpr int PER = 8;             // its elements per thread and block
 static_assert(SPLIT_WARPS * 32 * PER == TM * KB, "a block");
-static_assert(2 * PLANES * STAGES <= tc::SLOTS && STAGES <= tc::MAX_ASLOTS, "stages fit");
+static_assert(2 * PLANES * STAGES <= tc::SLOTS && STAGES <= tc::MAX_BSTAGES, "stages fit");
 
 struct Unit {
     int tile, kb0, kb1;
@@ -65,29 +65,30 @@ __device__ void producer(const SkinnyParams &p, tc::Smem &sm)
     int stage = 0;
     uint32_t lap = 0;
     bool ok = true;
+    bool skip = p.inject_timeout && blockIdx.x == 0;   // test hook: the first block never arrives
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit x = unit_of(p, u);
         const uint8_t *src = p.planes + (int64_t)x.kb0 * PLANES * PLANE_BYTES;
         for (int kb = x.kb0; kb < x.kb1; ++kb, src += PLANES * PLANE_BYTES) {
             ok = tc::mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
             if (!ok) break;
-            if (leader) {
-                tc::mbar_expect_tx(&sm.afull[stage], PLANES * bytes);
+            if (leader && !skip) {
+                tc::mbar_expect_tx(&sm.bfull[stage], PLANES * bytes);
                 for (int s = 0; s < PLANES; ++s)
                     tc::bulk_copy(big_plane(sm, stage, PLANES + s), src + s * PLANE_BYTES, bytes,
-                                  &sm.afull[stage]);
+                                  &sm.bfull[stage]);
             }
+            skip = false;
             if (++stage == STAGES) {
                 stage = 0;
                 ++lap;
             }
         }
     }
-    // no copy may outlive the CTA: every fill's phase completes only with the splitters'
-    // arrivals, which they make even when they give up
+    // no copy may outlive the CTA
     for (int i = 0; i < STAGES; ++i)
         if (i < stage || lap > 0)
-            tc::mbar_wait_drain(&sm.afull[i], (i < stage ? lap : lap - 1) & 1u, p.wait_ns);
+            tc::mbar_wait_drain(&sm.bfull[i], (i < stage ? lap : lap - 1) & 1u, p.wait_ns);
 }
 
 __device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc,
@@ -124,7 +125,9 @@ __device__ void issuer(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
             const uint32_t d = tmem + buf * 256;
             uint32_t accumulate = 0;
             for (int kb = k0; kb < k1; ++kb) {
-                ok = tc::mbar_wait(&sm.afull[stage], phase, sm, p.status, p.wait_ns);
+                // both operands' planes: the copies', and the splitting warps'
+                ok = tc::mbar_wait(&sm.bfull[stage], phase, sm, p.status, p.wait_ns) &&
+                     tc::mbar_wait(&sm.afull[stage], phase, sm, p.status, p.wait_ns);
                 if (!ok) break;
                 tc::tc_fence_after();
                 if (leader) {
@@ -190,6 +193,10 @@ struct Block {
     }
 };
 
+// A wait that gives up has raised the abort flag, and every later one returns at once; the unit
+// is run to its end all the same (its result is invalid, its accesses are the same), so that the
+// lanes of a warp stay together for the warp-wide instructions, and the warp leaves after it.  (A
+// vote of the lanes behind every drain's wait took 6 % of the kernel.)
 __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
 {
     const int t = threadIdx.x - 64, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -210,10 +217,9 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
         for (int c = 0; c < 32; ++c) acc[c] = 0.f;
         int chunks = 0;   // of this unit drained
         auto drain_to = [&](int want) {
-            for (; chunks < want && ok; ++chunks, ++drained) {
+            for (; chunks < want; ++chunks, ++drained) {
                 const uint32_t buf = drained & 1u;
-                ok = tc::mbar_wait(&sm.tfull[buf], (drained >> 1) & 1u, sm, p.status, p.wait_ns);
-                if (!ok) return;
+                ok &= tc::mbar_wait(&sm.tfull[buf], (drained >> 1) & 1u, sm, p.status, p.wait_ns);
                 tc::tc_fence_after();
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * 256 +
                                        (uint32_t)(part * cols);
@@ -245,16 +251,14 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
             src += step;
             left -= KB;
         }
-        for (int b0 = 0; b0 < len && ok; b0 += DEPTH) {
+        for (int b0 = 0; b0 < len; b0 += DEPTH) {
 #pragma unroll
             for (int d = 0; d < DEPTH; ++d) {
                 const int b = b0 + d;   // block within the unit
-                if (b >= len || !ok) break;
+                if (b >= len) break;
                 // a chunk is drained a block or two into the next, when its MMAs are through
                 if ((b & (p.chunk - 1)) == lag) drain_to(b / p.chunk);
-                if (!ok) break;
-                ok = tc::mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
-                if (!ok) break;
+                ok &= tc::mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
                 mine.store(big_plane(sm, stage, 0), v[d], high, low);
                 // the MMA reads these through the async proxy
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -269,7 +273,8 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
                 left -= KB;
             }
         }
-        if (ok) drain_to((len + p.chunk - 1) / p.chunk);
+        drain_to((len + p.chunk - 1) / p.chunk);
+        ok = __all_sync(0xffffffffu, ok) != 0;
         if (!ok) break;
         // partial sums of the unit: [small row][128 rows of the large operand]
         float *out = p.partial + ((int64_t)u * p.n16 + part * cols) * TM + quarter * 32 + lane;
@@ -279,9 +284,6 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
     }
     const bool bad = high >= tc::HIGH_BITS || low < tc::LOW_BITS - 1u;
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(p.gate, 1u);
-    if (!ok && lane == 0)
-        // let the producer's fills complete: it may have copied up to STAGES blocks more
-        for (int i = 0; i < STAGES; ++i) tc::mbar_arrive(&sm.afull[i]);
 }
 
 __global__ void __launch_bounds__(THREADS, 1) skinny_kernel(const SkinnyParams p)
@@ -292,7 +294,8 @@ __global__ void __launch_bounds__(THREADS, 1) skinny_kernel(const SkinnyParams p
     const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
         for (int i = 0; i < STAGES; ++i) {
-            tc::mbar_init(&sm.afull[i], 1 + SPLIT_WARPS);
+            tc::mbar_init(&sm.afull[i], SPLIT_WARPS);
+            tc::mbar_init(&sm.bfull[i], 1);
             tc::mbar_init(&sm.aempty[i], 1);
         }
         for (int i = 0; i < 2; ++i) {
@@ -322,6 +325,7 @@ __global__ void __launch_bounds__(THREADS, 1) skinny_kernel(const SkinnyParams p
     else
         splitter(p, sm, tmem);
     tc::tc_fence_before();
+    __syncwarp();
     __syncthreads();
     tc::tc_fence_after();
     if (warp == 1)

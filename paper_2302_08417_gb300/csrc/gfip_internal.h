@@ -120,6 +120,8 @@ template <typename T> struct GemmParams {
     unsigned long long *tile_next;   // epoch-tagged count of data-parallel tiles taken
     unsigned int *gate;              // nullable (FP32): the launch does nothing while the word is
                                      // zero, and clears it when it has run
+    unsigned long long wait_ns;      // FP32: budget of every mbarrier wait (nanoseconds)
+    int inject_timeout;              // FP32 test hook: CTA 0 withholds its first operand's arrival
 };
 
 // Parameters of the pack kernel of the pack-then-compute variant.
@@ -195,6 +197,7 @@ struct SkinnyParams {
     unsigned int *gate;      // set when an element is outside the range of the split
     unsigned int *status;
     unsigned long long wait_ns;
+    int inject_timeout;      // test hook: CTA 0 withholds its first copies
 };
 // Splits the small operand, runs the product and adds the k ranges into C (big_is_row: the large
 // operand's rows are C's rows), which is untouched when *gate is set.
@@ -236,7 +239,8 @@ cudaError_t launch_trsm_panel_f64(double *B, int64_t vstride, int64_t estride, i
 cudaError_t launch_trsm_panel_f32(float *B, int64_t vstride, int64_t estride, int nvec,
                                   const float *A, int64_t lda, int a_trans, int k0, int pw,
                                   int lower_t, int transpose_t, int unit, float *image,
-                                  unsigned int *status, cudaStream_t s);
+                                  unsigned int *status, unsigned long long wait_ns,
+                                  int inject_timeout, cudaStream_t s);
 size_t trsm_image_bytes(int pw);
 bool trsm_packs(int pw);
 

@@ -147,6 +147,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Smem &
     return false;
 }
 
+// The same wait by a whole converged warp, whose lanes go on or give up together: each lane sees
+// the timer and the abort flag at its own moment, and a lane that left alone would be missed by
+// the warp-wide instructions behind the wait.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, Smem &sm,
+                                               unsigned *status, unsigned long long budget_ns)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, sm, status, budget_ns)) != 0;
+}
+
 // The same wait, used while draining after an abort: ignores the abort flag and raises
 // nothing; returns when the budget runs out.
 __device__ __forceinline__ void mbar_wait_drain(uint64_t *bar, uint32_t parity,
@@ -468,6 +477,7 @@ __device__ __forceinline__ void f32_producer(const TcParams &p, Smem &sm)
     int stage = 0;
     uint32_t lap = 0;
     bool ok = true;
+    bool skip = p.inject_timeout && blockIdx.x == 0;   // test hook: the first block never arrives
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit x = unit_of(p, u);
         const uint8_t *a = p.pa + ((int64_t)x.i * p.kt + x.kb0) * F32_BYTES;
@@ -475,12 +485,13 @@ __device__ __forceinline__ void f32_producer(const TcParams &p, Smem &sm)
         for (int kb = x.kb0; kb < x.kb1; ++kb, a += F32_BYTES, b += F32_BYTES) {
             ok = mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
             if (!ok) break;
-            if (leader) {
+            if (leader && !skip) {
                 uint8_t *dst = sm.plane[stage * 2 * F32_PLANES];
                 mbar_expect_tx(&sm.afull[stage], 2 * F32_BYTES);
                 bulk_copy(dst, a, F32_BYTES, &sm.afull[stage]);
                 bulk_copy(dst + F32_BYTES, b, F32_BYTES, &sm.afull[stage]);
             }
+            skip = false;
             if (++stage == F32_STAGES) {
                 stage = 0;
                 ++lap;
@@ -704,7 +715,8 @@ template <int KIND> __device__ void epilogue(const TcParams &p, Smem &sm, uint32
                 KIND == KIND_F32 ? Group{2, 4, p.chunk} : group_of(g, p.planes);
             for (int k0 = x.kb0; k0 < x.kb1; k0 += q.chunk, ++chunks) {
                 const int buf = chunks % NBUF;
-                if (!mbar_wait(&sm.tfull[buf], (chunks / NBUF) & 1u, sm, p.status, p.wait_ns))
+                if (!mbar_wait_warp(&sm.tfull[buf], (chunks / NBUF) & 1u, sm, p.status,
+                                    p.wait_ns))
                     return;
                 tc_fence_after();
                 const uint32_t taddr =
@@ -863,6 +875,7 @@ template <int KIND> __global__ void __launch_bounds__(THREADS, 1) tc_kernel(cons
         epilogue<KIND>(p, sm, tmem);
     }
     tc_fence_before();
+    __syncwarp();
     __syncthreads();
     tc_fence_after();
     if (warp == 1)

@@ -1,6 +1,6 @@
 // gfip_testing.h -- test-only entry points of libgemmfip.so.  Not part of the public ABI
-// (include/gemmfip.h): nothing in the library's normal use calls them, and the only caller is
-// the failure-path test of the tensor-core FP64 emulation.
+// (include/gemmfip.h): nothing in the library's normal use calls them, and the only callers are
+// tests.
 #pragma once
 
 #include <stdint.h>
@@ -20,6 +20,13 @@ extern "C" {
  * tensor memory and returns; the context stays usable.  Nothing else is affected.
  * Returns GFIP_ERR_HANDLE for an invalid handle. */
 int gfip_debug_ozaki_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns);
+
+/* The same for the FP32 kernels with pipeline waits: the first CTA's first operand copy never
+ * arrives (tensor-core tile core, kernel for at most 128 rows or columns, warp-specialised FFMA
+ * core, TRSM panels of more than 96 unknowns), so its wait runs out: the call raises
+ * GFIP_STATUS_WAIT_TIMEOUT and its result is invalid (a TRSM panel's right-hand sides of that
+ * CTA stay as they are). */
+int gfip_debug_f32_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns);
 
 #ifdef __cplusplus
 }

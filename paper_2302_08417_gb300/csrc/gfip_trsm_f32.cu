@@ -36,7 +36,6 @@ constexpr int NV = 16;                       // right-hand sides per CTA
 constexpr int WARPS = 8;
 constexpr int XP = NV + 1;                   // pitch of the right-hand sides, one row per unknown
 constexpr unsigned STATUS_WAIT_TIMEOUT = 0x8u;           // mirrors GFIP_STATUS_WAIT_TIMEOUT
-constexpr unsigned long long WAIT_BUDGET_NS = 2000000000ull;
 
 // The packed panel of nb blocks, floats: diagonal entries [32 nb], their reciprocals [32 nb],
 // the diagonal blocks [nb][column][row], then each block's columns below it [column][row].
@@ -125,8 +124,9 @@ __device__ __forceinline__ void fetch(float *dst, const float *src, int n, unsig
         : "memory");
 }
 
-// Waits for a phase of *bar; false if it gave up after WAIT_BUDGET_NS.
-__device__ __forceinline__ bool arrived(unsigned long long *bar, uint32_t parity)
+// Waits for a phase of *bar; false if it gave up after budget_ns.
+__device__ __forceinline__ bool arrived(unsigned long long *bar, uint32_t parity,
+                                        unsigned long long budget_ns)
 {
     unsigned long long t0 = 0;
     for (long long it = 0; it < (1ll << 32); ++it) {
@@ -142,7 +142,7 @@ __device__ __forceinline__ bool arrived(unsigned long long *bar, uint32_t parity
             unsigned long long t;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
             if (t0 == 0) t0 = t;
-            if (t - t0 > WAIT_BUDGET_NS) break;
+            if (t - t0 > budget_ns) break;
         }
     }
     return false;
@@ -292,7 +292,8 @@ static_assert(SELF_BLOCKS <= 3 && SELF_BLOCKS * BLK <= WARPS * 32, "two column b
 
 __global__ void __launch_bounds__(WARPS * 32, 1)
     panel_kernel(float *B, int64_t vstride, int64_t estride, int nvec, const Panel p,
-                 const float *image, unsigned int *status)
+                 const float *image, unsigned int *status, unsigned long long wait_ns,
+                 int inject_timeout)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -318,7 +319,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (!self && !plain) {
-            fetch(sm.head, image, head_floats(nb), &sm.full[2]);
+            if (!(inject_timeout && blockIdx.x == 0))   // test hook: its first copy never starts
+                fetch(sm.head, image, head_floats(nb), &sm.full[2]);
             fetch_columns(0);
             fetch_columns(1);
         }
@@ -332,9 +334,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     move_sides<false>(p, B, vstride, estride, nvec, nb * BLK, sm);
     __syncthreads();
     const bool staged = self || plain;
-    bool ok = staged || arrived(&sm.full[2], 0);
+    // all threads go on or give up together
+    bool ok = __syncthreads_and(staged || arrived(&sm.full[2], 0, wait_ns));
     if (warp == 0 && ok) solve_block(sm, nb, 0);
-    ok = __syncthreads_and(ok);
+    __syncthreads();
     int bk = 0;
     for (; bk + 1 < nb && ok; ++bk) {
         float2 nx[BLK];
@@ -344,7 +347,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
             const float v = -x[j * XP];
             nx[j] = make_float2(v, v);
         }
-        ok = staged || arrived(&sm.full[bk & 1], (bk >> 1) & 1);
+        ok = staged || arrived(&sm.full[bk & 1], (bk >> 1) & 1, wait_ns);
         const int units = (nb - 1 - bk) * (BLK / 16);
         if (warp < 2) {
             update_rows(sm, nb, bk, warp, nx);   // the next block's rows
@@ -366,7 +369,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
         // a copy never arrived: leave B as it is, and no copy behind (fetched, not awaited yet)
         if (tid == 0) {
             atomicOr(status, STATUS_WAIT_TIMEOUT);
-            for (int b = bk; b < bk + 2 && b + 1 < nb; ++b) arrived(&sm.full[b & 1], (b >> 1) & 1);
+            for (int b = bk; b < bk + 2 && b + 1 < nb; ++b)
+                arrived(&sm.full[b & 1], (b >> 1) & 1, wait_ns);
         }
         return;
     }
@@ -389,7 +393,8 @@ size_t trsm_image_bytes(int pw)
 cudaError_t launch_trsm_panel_f32(float *B, int64_t vstride, int64_t estride, int nvec,
                                   const float *A, int64_t lda, int a_trans, int k0, int pw,
                                   int lower_t, int transpose_t, int unit, float *image,
-                                  unsigned int *status, cudaStream_t s)
+                                  unsigned int *status, unsigned long long wait_ns,
+                                  int inject_timeout, cudaStream_t s)
 {
     using namespace trsm32;
     if (nvec <= 0 || pw <= 0) return cudaSuccess;
@@ -420,8 +425,8 @@ cudaError_t launch_trsm_panel_f32(float *B, int64_t vstride, int64_t estride, in
         image = nullptr;
     else
         pack_kernel<<<nb * (nb + 1) / 2, 256, 0, s>>>(p, nb, image);
-    panel_kernel<<<(nvec + NV - 1) / NV, WARPS * 32, sizeof(Smem), s>>>(B, vstride, estride, nvec,
-                                                                        p, image, status);
+    panel_kernel<<<(nvec + NV - 1) / NV, WARPS * 32, sizeof(Smem), s>>>(
+        B, vstride, estride, nvec, p, image, status, wait_ns, inject_timeout);
     return cudaGetLastError();
 }
 

@@ -70,7 +70,6 @@ constexpr int STAGES = Cfg::STAGES;
 constexpr int TILE_FLOATS = 128 * 32;
 constexpr int TILE_BYTES = TILE_FLOATS * 4;    // one operand tile, packed or staged (16 KB)
 constexpr unsigned int STATUS_WAIT_TIMEOUT = 0x8u;       // mirrors GFIP_STATUS_WAIT_TIMEOUT
-constexpr unsigned long long WAIT_BUDGET_NS = 2000000000ull;
 constexpr long long WAIT_POLLS = 1ll << 40;              // the time budget ends every wait
 
 // Float offset of element (x, kk) of a tile in the swizzled layout.
@@ -146,7 +145,7 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity)
 // Waits for the phase of the given parity; gives up after the budget or when another role
 // has aborted.  A timeout sets the abort flag and the status bit.
 __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, uint32_t parity, Smem &sm,
-                                          unsigned int *status)
+                                          unsigned int *status, unsigned long long budget_ns)
 {
     const uint32_t a = smem_addr(bar);
     if (mbar_try(a, parity)) return true;
@@ -154,21 +153,32 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, uint32_t pari
     for (long long it = 0; it < WAIT_POLLS; ++it) {
         if (mbar_try(a, parity)) return true;
         if (aborted(sm)) return false;
-        if ((it & 63) == 63 && global_ns() - t0 > WAIT_BUDGET_NS) break;
+        if ((it & 63) == 63 && global_ns() - t0 > budget_ns) break;
     }
     *(volatile int *)&sm.abort = 1;
     atomicOr(status, STATUS_WAIT_TIMEOUT);
     return false;
 }
 
+// The same wait by a whole warp, whose lanes go on or give up together: each lane sees the timer
+// and the abort flag at its own moment, and a lane that left alone would be missed by the
+// warp-wide instructions behind the wait.
+__device__ __forceinline__ bool mbar_wait_warp(unsigned long long *bar, uint32_t parity, Smem &sm,
+                                               unsigned int *status,
+                                               unsigned long long budget_ns)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, sm, status, budget_ns)) != 0;
+}
+
 // The same wait while draining after an abort: ignores the flag, raises nothing.
-__device__ __forceinline__ void mbar_wait_drain(unsigned long long *bar, uint32_t parity)
+__device__ __forceinline__ void mbar_wait_drain(unsigned long long *bar, uint32_t parity,
+                                                unsigned long long budget_ns)
 {
     const uint32_t a = smem_addr(bar);
     const unsigned long long t0 = global_ns();
     for (long long it = 0; it < WAIT_POLLS; ++it) {
         if (mbar_try(a, parity)) return;
-        if ((it & 63) == 63 && global_ns() - t0 > WAIT_BUDGET_NS) return;
+        if ((it & 63) == 63 && global_ns() - t0 > budget_ns) return;
     }
 }
 
@@ -216,6 +226,19 @@ __device__ __forceinline__ void fence_proxy_shared()
 __device__ __forceinline__ void math_barrier(int ring)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(1 + ring), "n"(MATH_THREADS) : "memory");
+}
+
+// The same barrier; true if ok holds in all of the warpgroup's threads.
+__device__ __forceinline__ bool math_all(int ring, bool ok)
+{
+    uint32_t all;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n"
+        " selp.u32 %0, 1, 0, q;\n}"
+        : "=r"(all)
+        : "r"(ok ? 1u : 0u), "r"(1 + ring), "n"(MATH_THREADS)
+        : "memory");
+    return all != 0;
 }
 
 // The segments one (virtual) CTA g runs, in order: whole tiles of the data-parallel waves,
@@ -381,7 +404,7 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
             const int st = static_cast<int>(d % STAGES);
             if (m.prod) {
                 if (!mbar_wait(&rg.full[st], static_cast<uint32_t>((d / STAGES) & 1), sm,
-                               p.status)) {
+                               p.status, p.wait_ns)) {
                     ok = false;
                     return;
                 }
@@ -400,7 +423,8 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
         SegCursor cur;
         cur.start(p, g);
         Segment sg;
-        while (ok && !aborted(sm) && cur.next(p, sg)) {
+        bool withhold = p.inject_timeout && g == 0 && !OPB;   // test hook: the first k-block
+        while (__all_sync(0xffffffffu, ok && !aborted(sm)) && cur.next(p, sg)) {
             const int panel = OPB ? sg.j : sg.i;
             const int other = OPB ? sg.i : sg.j;
             // a panel that no later tile reuses is neither packed nor looked up (reused_a/_b)
@@ -420,8 +444,8 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
             for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
                 const int st = static_cast<int>(q % STAGES);
                 if (q >= STAGES &&
-                    !mbar_wait(&rg.empty[st], static_cast<uint32_t>(((q / STAGES) - 1) & 1), sm,
-                               p.status)) {
+                    !mbar_wait_warp(&rg.empty[st], static_cast<uint32_t>(((q / STAGES) - 1) & 1),
+                                    sm, p.status, p.wait_ns)) {
                     ok = false;
                     break;
                 }
@@ -442,7 +466,9 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
                         }
                     }
                     // this lane's arrival, with the copy-engine bytes the stage waits for
-                    mbar_arrive_expect_tx(&rg.full[st], d == 1 ? TILE_BYTES : 0);
+                    if (!withhold || d == 1)
+                        mbar_arrive_expect_tx(&rg.full[st], d == 1 ? TILE_BYTES : 0);
+                    withhold = false;
                     if (d == 1) bulk_load(buf(st), slot(panel, kb), TILE_BYTES, &rg.full[st]);
                 }
                 d = __shfl_sync(0xffffffffu, d, 0);
@@ -486,7 +512,8 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
             asm volatile("cp.async.wait_all;" ::: "memory");
             if (lane == 0)
                 for (long long d = q - 1; d >= 0 && d >= q - STAGES; --d)
-                    mbar_wait_drain(&rg.full[d % STAGES], static_cast<uint32_t>((d / STAGES) & 1));
+                    mbar_wait_drain(&rg.full[d % STAGES], static_cast<uint32_t>((d / STAGES) & 1),
+                                    p.wait_ns);
         }
     }
 
@@ -707,8 +734,14 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
         cur.start(p, g);
         Segment sg;
         bool ok = true;
-        while (ok && cur.next(p, sg)) {
+        // a warp that gave up still meets its warpgroup at every split segment
+        while (cur.next(p, sg)) {
             const int i = sg.i, j = sg.j;
+            const bool whole = sg.kb0 == 0 && sg.kb1 == p.kt;
+            if (!ok) {
+                if (!whole) math_all(ring, false);
+                continue;
+            }
 #pragma unroll
             for (int ii = 0; ii < TM; ++ii)
 #pragma unroll
@@ -724,10 +757,8 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
                 }
             }
             for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-                if (!mbar_wait(&rg.full[st], ph, sm, p.status)) {
-                    ok = false;
-                    break;
-                }
+                ok = mbar_wait_warp(&rg.full[st], ph, sm, p.status, p.wait_ns);
+                if (!ok) break;
                 compute(rg.a[st], rg.b[st], acc, tx, ty);
                 __syncwarp();
                 if ((tid & 31) == 0) mbar_arrive(&rg.empty[st]);
@@ -736,11 +767,12 @@ template <bool ACONTIG, bool BCONTIG> struct WsKernel {
                     ph ^= 1u;
                 }
             }
-            if (!ok) break;
-            if (sg.kb0 == 0 && sg.kb1 == p.kt)
-                epilogue(p, i, j, tid, acc);
-            else
-                fixup(p, rg, ring, g, sg.t, i, j, sg.slot, acc, epoch, tid);
+            if (whole) {
+                if (ok) epilogue(p, i, j, tid, acc);
+            } else {
+                ok = math_all(ring, ok);
+                if (ok) fixup(p, rg, ring, g, sg.t, i, j, sg.slot, acc, epoch, tid);
+            }
         }
     }
 };

@@ -76,6 +76,7 @@ SIGNATURES = {
     "gfip_sgemm_grouped_plan": (_int, [_ptr, _int] + [_ptr] * 15 + [_i64]),
     "gfip_dgemm_ozaki": (_int, _GEMM_D + [_int]),
     "gfip_debug_ozaki_timeout": (_int, [_ptr, _int, ctypes.c_uint64]),
+    "gfip_debug_f32_timeout": (_int, [_ptr, _int, ctypes.c_uint64]),
     "gfip_syrk_workspace_size": (_sz, [_ptr, _chr, _chr, _i64, _i64, _int]),
     "gfip_dsyrk": (_int, [_ptr, _chr, _chr, _i64, _i64, _dbl, _ptr, _i64, _dbl, _ptr, _i64]),
     "gfip_ssyrk": (_int, [_ptr, _chr, _chr, _i64, _i64, _flt, _ptr, _i64, _flt, _ptr, _i64]),
@@ -233,6 +234,12 @@ def gfip_debug_ozaki_timeout(handle, enable: bool, wait_ns: int = 0) -> int:
     """Test hook: later gfip_dgemm_ozaki calls withhold one operand copy in the first CTA so
     that its bounded wait (wait_ns; 0 = the 2 s default) runs out."""
     return load().gfip_debug_ozaki_timeout(handle, int(bool(enable)), int(wait_ns))
+
+
+def gfip_debug_f32_timeout(handle, enable: bool, wait_ns: int = 0) -> int:
+    """Test hook (declared in csrc/gfip_testing.h, not in the public header): makes the first
+    CTA's first pipeline wait of the FP32 kernels run out."""
+    return load().gfip_debug_f32_timeout(handle, int(bool(enable)), int(wait_ns))
 
 
 def gfip_syrk_workspace_size(handle, uplo, trans, n, k, elem_bytes) -> int:
