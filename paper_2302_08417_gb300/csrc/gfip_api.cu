@@ -54,6 +54,7 @@ struct Handle {
     int oz_inject = 0;                             // test hook (gfip_debug_ozaki_timeout)
     unsigned long long f32_wait_ns = kF32WaitNs;   // budget of the FP32 kernels' waits
     int f32_inject = 0;                            // test hook (gfip_debug_f32_timeout)
+    int route = GFIP_ROUTE_AUTO;                   // test hook (gfip_debug_route)
     int last_launches = 0;
     int last_grid = 0;
     int bps_f64 = 0;
@@ -263,7 +264,7 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
 {
     TcPlan t;
     if (sizeof(T) != 4 || k > kTcMaxK || k < kTcMinK) return t;
-    t.use = true;
+    t.use = h->route != GFIP_ROUTE_CORE;
     t.mt = static_cast<int>((m + 127) / 128);
     t.nt = static_cast<int>((n + 127) / 128);
     t.kt = static_cast<int>((k + 31) / 32);
@@ -293,7 +294,7 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
         const int64_t rounds = ((int64_t)t.tiles * t.splits + h->sms - 1) / h->sms;
         const double ns = 17000 + (double)rounds * ((t.kt + t.splits - 1) / t.splits) *
                                       (600 + 3.2 * n16) + 1000.0 * t.splits;
-        if (ns < t.ns) {
+        if (h->route == GFIP_ROUTE_SKINNY || (ns < t.ns && h->route != GFIP_ROUTE_TENSOR)) {
             t.skinny = true;
             t.n16 = n16;
             t.ns = ns;
@@ -332,6 +333,7 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
 template <typename T>
 bool use_small(const Handle *h, const TcPlan &tc, int64_t m, int64_t n, int64_t k, int tri)
 {
+    if (h->route != GFIP_ROUTE_AUTO) return h->route == GFIP_ROUTE_SMALL;
     const double work = (double)m * n * k, part = tri ? 0.5 : 1.0;
     if (sizeof(T) == 8)
         return work <= (double)(1ll << 35) && (k > 64 || (double)m * n <= (double)(1 << 24));
@@ -1089,6 +1091,15 @@ int gfip_debug_f32_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns)
     if (h == nullptr) return GFIP_ERR_HANDLE;
     h->f32_inject = enable ? 1 : 0;
     h->f32_wait_ns = wait_ns ? wait_ns : kF32WaitNs;
+    return GFIP_OK;
+}
+
+int gfip_debug_route(gfip_handle_t handle, int route)
+{
+    Handle *h = get(handle);
+    if (h == nullptr) return GFIP_ERR_HANDLE;
+    if (route < GFIP_ROUTE_AUTO || route > GFIP_ROUTE_SKINNY) return GFIP_ERR_ARG;
+    h->route = route;
     return GFIP_OK;
 }
 

@@ -28,6 +28,17 @@ int gfip_debug_ozaki_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns)
  * CTA stay as they are). */
 int gfip_debug_f32_timeout(gfip_handle_t handle, int enable, uint64_t wait_ns);
 
+/* Sends this handle's later products (GEMM, SYRK, TRMM, TRSM updates) to one path wherever that
+ * path can compute them, whatever their size: the fused-in-packing core alone, the small
+ * kernels, the tensor cores from planes, or the tensor cores' kernel for at most 128 rows or
+ * columns (FP32; the core, or the planes, where it cannot be used). */
+#define GFIP_ROUTE_AUTO 0
+#define GFIP_ROUTE_CORE 1
+#define GFIP_ROUTE_SMALL 2
+#define GFIP_ROUTE_TENSOR 3
+#define GFIP_ROUTE_SKINNY 4
+int gfip_debug_route(gfip_handle_t handle, int route);
+
 #ifdef __cplusplus
 }
 #endif

@@ -77,6 +77,7 @@ SIGNATURES = {
     "gfip_dgemm_ozaki": (_int, _GEMM_D + [_int]),
     "gfip_debug_ozaki_timeout": (_int, [_ptr, _int, ctypes.c_uint64]),
     "gfip_debug_f32_timeout": (_int, [_ptr, _int, ctypes.c_uint64]),
+    "gfip_debug_route": (_int, [_ptr, _int]),
     "gfip_syrk_workspace_size": (_sz, [_ptr, _chr, _chr, _i64, _i64, _int]),
     "gfip_dsyrk": (_int, [_ptr, _chr, _chr, _i64, _i64, _dbl, _ptr, _i64, _dbl, _ptr, _i64]),
     "gfip_ssyrk": (_int, [_ptr, _chr, _chr, _i64, _i64, _flt, _ptr, _i64, _flt, _ptr, _i64]),
@@ -240,6 +241,16 @@ def gfip_debug_f32_timeout(handle, enable: bool, wait_ns: int = 0) -> int:
     """Test hook (declared in csrc/gfip_testing.h, not in the public header): makes the first
     CTA's first pipeline wait of the FP32 kernels run out."""
     return load().gfip_debug_f32_timeout(handle, int(bool(enable)), int(wait_ns))
+
+
+# paths of gfip_debug_route (GFIP_ROUTE_* of csrc/gfip_testing.h)
+ROUTES = {"auto": 0, "core": 1, "small": 2, "tensor": 3, "skinny": 4}
+
+
+def gfip_debug_route(handle, route: str) -> int:
+    """Test hook (declared in csrc/gfip_testing.h, not in the public header): sends the handle's
+    products to one path wherever that path can compute them."""
+    return load().gfip_debug_route(handle, ROUTES[route])
 
 
 def gfip_syrk_workspace_size(handle, uplo, trans, n, k, elem_bytes) -> int:
