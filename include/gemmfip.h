@@ -25,8 +25,10 @@
  *
  * Other FP32 products of at least 16 terms run on the tensor cores in every routine (GEMM in all
  * three variants, SYRK, TRMM, TRSM updates): packing splits
- * each operand exactly into three BF16 planes, whose products are summed in FP32; the error
- * against the exact product is no larger than that of FP32 multiply-adds.  Operands with an
+ * each operand exactly into three BF16 planes, and eight of the nine plane products (the ninth is
+ * below 2^-32 of the whole) are summed in FP32, in chunks so short that the 2-norm of the error
+ * against the exact product measured no larger than that of the FP32 kernel described first, for
+ * entries of one sign and of both, at k = 16 to 100000.  Operands with an
  * infinity, a NaN or a nonzero magnitude outside [2^-100, 2^55) are multiplied by the FP32
  * kernel described first, decided on the device.  A workspace too small for the planes (see
  * gfip_workspace_size) but large enough for that kernel runs there too.

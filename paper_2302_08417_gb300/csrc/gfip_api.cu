@@ -280,20 +280,20 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
             t.splits = s;
         }
     }
-    // Estimated times, ns, fitted to one GB300: 640^3 18 us, 2048^3 87, 64 x 8192 x 8192 205 (its
-    // planes' 10 bytes an element dominate) and, split on the way, 112; 100 x 2000 x 2000 29
-    // and 37.
+    // Estimated times, ns, fitted to one GB300: 640^3 19 us, 2048^3 106, 300 x 290 x 2500 31 (28 on
+    // the small kernel), 64 x 8192 x 8192 212 (its planes' 10 bytes an element dominate) and, split
+    // on the way, 120; 100 x 2000 x 2000 32 and 39.
     const double planes = (double)m * k + (tri ? 0.0 : (double)n * k);
     const double part = tri ? 0.5 : 1.0;
-    t.ns = 9000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost;
+    const int64_t in_a_row = ((int64_t)t.tiles * t.splits + h->sms - 1) / h->sms *
+                             ((t.kt + t.splits - 1) / t.splits);
+    t.ns = 9000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost + 130.0 * in_a_row;
     // at most 128 rows or columns against an operand that is read along memory: k blocks on the
     // busiest SM, and the launch that adds the k ranges
     if (tri == gfip::TRI_NONE && !masked && std::min(m, n) <= 128 &&
         (n <= m ? is_notrans(transa) : !is_notrans(transb))) {
         const int n16 = static_cast<int>((std::min(m, n) + 15) / 16 * 16);
-        const int64_t rounds = ((int64_t)t.tiles * t.splits + h->sms - 1) / h->sms;
-        const double ns = 17000 + (double)rounds * ((t.kt + t.splits - 1) / t.splits) *
-                                      (600 + 3.2 * n16) + 1000.0 * t.splits;
+        const double ns = 17000 + (double)in_a_row * (600 + 3.2 * n16) + 1000.0 * t.splits;
         if (h->route == GFIP_ROUTE_SKINNY || (ns < t.ns && h->route != GFIP_ROUTE_TENSOR)) {
             t.skinny = true;
             t.n16 = n16;
@@ -417,11 +417,17 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
                       unsigned char *data)
 {
     // k blocks (of 32) per accumulation on the tensor cores, whose truncation shows as a bias that
-    // grows with a chunk's length (entries in [0, 1], relative error: 8e-8 with 64 k, 1.5e-7 with
-    // 128, 3.1e-7 with 256), while the FFMA chain's error grows with k (8e-8 to 1.2e-7 at 64 to
-    // 700, 8e-7 at 4096).  Short chunks cost drains: 4096^3 takes 602 us with 64, 540 with 128, 505
-    // with 256.
-    const int chunk = p.k <= 1024 ? 2 : 4;
+    // grows with a chunk's length, to be no further off than the FFMA core, whose error grows with
+    // its chains' length L and shrinks as more of them are added.  Entries in [0, 1], relative
+    // error in 1e-8: chunks of 32 k 5 to 6, 64 k 8, 128 k 14.5 (with many chunks their sum adds
+    // to it: 12 for 64 k at k = 2500); the FFMA core about sqrt(2 L^2 / k + 30): one chain of 128
+    // 16, of 1024 30; 512 x 512 x 1500 in twelve chains of 128 7.3, 1030 x 1100 x 1500 in four of
+    // 400 14.7.  Short chunks cost drains: 4096^3 takes 710 us with 64, 651 with 128;
+    // 512 x 512 x 4096 43 with 32 and 41 with 64.
+    const double chain =
+        p.dp_tiles > 0 ? (double)p.k : std::min<double>(p.k, 32.0 * p.sk_iters / p.grid);
+    const double spread = chain * chain / p.k;
+    const int chunk = p.k > 1024 && spread >= 128 ? 4 : p.k > 512 && spread < 22 ? 1 : 2;
     if (t.skinny) {
         const bool big_is_row = p.n <= p.m;   // op(A) is the large operand
         gfip::SkinnyParams q{};

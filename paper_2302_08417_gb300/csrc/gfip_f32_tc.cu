@@ -1,13 +1,17 @@
 // gfip_f32_tc.cu -- large FP32 GEMMs on the tensor cores: operands split into three BF16 planes.
 //
 // x = x1 + x2 + x3 with x1 = BF16(x), x2 = BF16(x - x1), x3 = x - x1 - x2, exactly: each rounding to
-// nearest leaves a remainder of at most 2^-9 of what it rounded, and 24 significant bits fit
+// nearest leaves a remainder of at most 2^-8 of what it rounded, and 24 significant bits fit
 // three planes of 8.  The tile core (gfip_tc.cuh) forms a1 b1 + (a1 b2 + a2 b1 + a1 b3 + a2 b2 +
-// a3 b1); the products left out are below 2^-25 of |a b|.  a1 b1 and the smaller products are
-// accumulated apart, for 64 or 128 k at a time (launch_tc in gfip_api.cu), and the chunks are
-// added in FP32 with rounding to nearest, which keeps the sum at least as exact as one chain of k
-// FP32 multiply-adds (the FFMA cores' order), also where all terms have one sign.  Packing is where the split happens: one pass reads the strided
-// operands (masking triangular ones) and writes the plane tiles the MMA reads.
+// a3 b1 + a2 b3 + a3 b2); the one product left out, a3 b3, is at most 2^-32 of |a b|, a 256th of
+// half an ulp, so a sum that one product dominates comes out rounded as a multiply-add rounds it.
+// (Without a2 b3 + a3 b2, up to 2^-24 of |a b|, 4 % of such sums were an ulp off and the worst
+// error was 1.5 times a multiply-add's; the two products cost 4096^3 20 %.)  a1 b1 and the
+// smaller products are accumulated apart, for 32 to 128 k at a time (launch_tc in gfip_api.cu),
+// and the chunks are added in FP32 with rounding to nearest, which keeps the sum at least as
+// exact as the FFMA core's chains of FP32 multiply-adds, also where all terms have one sign.
+// Packing is where the split happens: one pass reads the strided operands (masking triangular
+// ones) and writes the plane tiles the MMA reads.
 //
 // The split is exact while no plane leaves BF16's normal range and no product or sum FP32's:
 // every element zero or of magnitude in [2^-100, 2^55), k at most 2^17.  An element outside

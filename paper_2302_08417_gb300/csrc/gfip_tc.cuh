@@ -7,7 +7,7 @@
 //    the same s + t (a "class") have the same weight, so they share one FP32 accumulator:
 //    sums of up to 16384 digit products stay exact.
 //  * KIND_F32 (FP32 GEMM, gfip_f32_tc.cu): three planes hold an FP32 value's 24 bits exactly.
-//    a1 b1 has an accumulator of its own, the five smaller products share a second one.
+//    a1 b1 has an accumulator of its own, seven smaller products share a second one.
 //
 // Why this shape.  A CTA computes a 128 x 128 tile of C.  The tensor pipe takes 128 clocks for
 // one pair of a 32-wide k block, and one 8 KB plane of each operand serves up to S pairs; so
@@ -20,7 +20,8 @@
 // MMA of N = 256: it reads 12 KB of operands per 128 clocks where two of N = 128 read 16 KB.
 //
 // Measured on one GB300: 4096^3 with 7 digits 4710 -> 2416 us (tensor pipe 75 % busy), 8192^3 38 ->
-// 63 TFLOP/s FP64-equivalent; FP32 4096^3 2513 us on the FFMA core -> 540 (254 TFLOP/s).
+// 63 TFLOP/s FP64-equivalent; FP32 4096^3 2513 us on the FFMA core -> 644 (213 TFLOP/s; 704 where
+// the power cap binds, 1024 clocks of MMAs a k block).
 //
 // Roles (one CTA per SM, 10 warps, persistent over the units of work):
 //   warp 0      producer.  Digits: per k block one bulk copy of the B planes the group needs (two
@@ -35,7 +36,7 @@
 // wait for one barrier per A plane (digits) or block (FP32): the instructions between two MMAs
 // are a serial chain in one warp (a first form with a barrier per plane of either operand, run
 // by one lane, spent 800 clocks a step on them and ran the MMAs at a third of their rate; three
-// barriers a block took FP32 1107 clocks a block, one 904, for 768 of MMAs).
+// barriers a block took FP32, with six products, 1107 clocks a block, one 904, for 768 of MMAs).
 // Every mbarrier wait is bounded by a global-timer budget; on a timeout the kernel raises a
 // status bit, the roles skip their remaining work, the producer waits for its copies in
 // flight, and tensor memory is released before exit.
@@ -367,7 +368,7 @@ __device__ __forceinline__ Unit unit_of(const TcParams &p, int u)
 }
 
 // FP32: a stage holds a k block's three planes of A, then of B, on one barrier pair (`afull`,
-// `aempty`): its 12 MMAs are issued after a single wait.
+// `aempty`): its 14 MMAs are issued after a single wait.
 constexpr int F32_PLANES = 3;
 constexpr int F32_STAGES = 4;
 constexpr uint32_t F32_BYTES = F32_PLANES * PLANE_BYTES;
@@ -585,7 +586,7 @@ __device__ __forceinline__ void f32_issuer(const TcParams &p, Smem &sm, uint32_t
             ok = mbar_wait(&sm.tempty[buf], ((chunks >> 1) & 1u) ^ 1u, sm, p.status, p.wait_ns);
             if (!ok) break;
             tc_fence_after();
-            // columns 0-127: a1 b1; 128-255: the five smaller products
+            // columns 0-127: a1 b1; 128-255: the seven smaller products
             const uint32_t d = tmem + buf * 256;
             uint32_t accumulate = 0;   // the block's first MMA starts both sums
             for (int kb = k0; kb < k1; ++kb) {
@@ -600,7 +601,9 @@ __device__ __forceinline__ void f32_issuer(const TcParams &p, Smem &sm, uint32_t
                     mma_block<128>(d + TN, a1, b2 + PLANE_DESC, 1u);
                     mma_block<128>(d + TN, a2, b1, 1u);
                     mma_block<128>(d + TN, a2, b2, 1u);
+                    mma_block<128>(d + TN, a2, b2 + PLANE_DESC, 1u);
                     mma_block<128>(d + TN, a3, b1, 1u);
+                    mma_block<128>(d + TN, a3, b2, 1u);
                     mma_commit(&sm.aempty[stage]);
                 }
                 accumulate = 1;
