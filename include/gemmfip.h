@@ -29,7 +29,7 @@
  * below 2^-32 of the whole) are summed in FP32, in chunks so short that the 2-norm of the error
  * against the exact product measured no larger than that of the FP32 kernel described first, for
  * entries of one sign and of both, at k = 16 to 100000.  Operands with an
- * infinity, a NaN or a nonzero magnitude outside [2^-100, 2^55) are multiplied by the FP32
+ * infinity, a NaN or a nonzero magnitude outside [2^-100, 2^47) are multiplied by the FP32
  * kernel described first, decided on the device.  A workspace too small for the planes (see
  * gfip_workspace_size) but large enough for that kernel runs there too.
  *

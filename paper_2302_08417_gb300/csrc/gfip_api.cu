@@ -453,7 +453,8 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
                                        big_is_row ? p.b_contig_n : p.a_contig_m,
                                        1,
                                        0,
-                                       data + t.off_a};
+                                       data + t.off_a,
+                                       256.f};
         return gfip::launch_f32_skinny(q, small, p.C, p.ldc, big_is_row ? 1 : 0, p.alpha, p.beta,
                                        h->sms, h->stream);
     }
@@ -483,8 +484,10 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
     q.status = p.status;
     q.wait_ns = p.wait_ns;
     q.inject_timeout = p.inject_timeout;
-    const gfip::F32SplitArgs a{p.A, p.lda, p.m, p.a_contig_m, t.mt, p.tmask_a, data + t.off_a};
-    gfip::F32SplitArgs b{p.B, p.ldb, p.n, p.b_contig_n, t.nt, p.tmask_b, data + t.off_b};
+    const gfip::F32SplitArgs a{p.A, p.lda, p.m, p.a_contig_m, t.mt, p.tmask_a, data + t.off_a,
+                               16.f};
+    gfip::F32SplitArgs b{p.B, p.ldb, p.n, p.b_contig_n, t.nt, p.tmask_b, data + t.off_b,
+                         16.f};
     if (p.tri != gfip::TRI_NONE) b.row_blocks = 0;   // both roles read the planes of A
     return gfip::launch_f32_tc(q, a, b, p.k, p.gate, h->sms, h->stream);
 }

@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(256) add_kernel(const SkinnyParams p, float *C
         const int s = big_is_row ? e >> 5 : e - b * small_rows;
         if (b0 + b >= p.rows) continue;
         float *c = C + (big_is_row ? (b0 + b) + (int64_t)s * ldc : s + (int64_t)(b0 + b) * ldc);
-        const float v = alpha * tile[s][b];
+        const float v = alpha * (tile[s][b] * tc::F32_UNSCALE);
         *c = read_c ? fmaf(beta, *c, v) : v;
     }
 }

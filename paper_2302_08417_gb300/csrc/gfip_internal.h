@@ -172,6 +172,7 @@ struct F32SplitArgs {
     int row_blocks;   // 0: nothing to split (SYRK: B's planes are A's)
     int mask;         // triangular operand (TRMM), 0 = dense; see TriMask
     uint8_t *planes;
+    float scale;      // power of two: the planes are those of the scaled elements
 };
 // Splits both operands and launches the tile core; an element outside the range of the split
 // sets *gate (which also makes the tile core do nothing).

@@ -375,9 +375,11 @@ constexpr uint32_t F32_BYTES = F32_PLANES * PLANE_BYTES;
 static_assert(F32_STAGES * 2 * F32_PLANES <= SLOTS && F32_STAGES <= MAX_ASLOTS, "stages fit");
 
 // The range in which an FP32 element's split into three BF16 planes is exact and safe
-// (gfip_f32_tc.cu): zero, or a magnitude in [2^-100, 2^55).
+// (gfip_f32_tc.cu): zero, or a magnitude in [2^-100, 2^47).  The operands' planes are those of
+// the elements times powers of two that multiply to 1 / F32_UNSCALE.
 constexpr uint32_t LOW_BITS = (127u - 100u) << 23;   // 2^-100
-constexpr uint32_t HIGH_BITS = (127u + 55u) << 23;   // 2^55
+constexpr uint32_t HIGH_BITS = (127u + 47u) << 23;   // 2^47
+constexpr float F32_UNSCALE = 1.f / 256.f;
 
 __device__ __forceinline__ bool outside_split(float x)
 {
@@ -815,7 +817,7 @@ template <int KIND> __device__ void epilogue(const TcParams &p, Smem &sm, uint32
                 const bool in = static_cast<uint32_t>(col - first) < count;
                 T v;
                 if constexpr (KIND == KIND_F32) {
-                    v = alpha * acc[g * W + i];
+                    v = alpha * (acc[g * W + i] * F32_UNSCALE);
                     if (read_c) v = fmaf(beta, cv[i], v);
                 } else {
                     v = alpha * scale2((double)acc[g * W + i], er + (in ? p.eb[col] : 0));

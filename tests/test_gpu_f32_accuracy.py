@@ -74,3 +74,18 @@ def test_error_no_larger_than_the_cores(multiply, route, m, n, sign):
         err = {r: np.linalg.norm(multiply(r, A, B) - want) for r in ("core", route)}
         assert err[route] <= err["core"], (k, err[route] / np.linalg.norm(want),
                                            err["core"] / np.linalg.norm(want))
+
+
+@pytest.mark.parametrize("ea,eb", [(-60, -60), (-65, -65), (-70, -70), (-99, -30), (-90, -50),
+                                   (-99, 46)])
+@pytest.mark.parametrize("route,m,n,k", [("tensor", 700, 690, 660), ("skinny", 2000, 100, 1499)])
+def test_small_products_lose_no_more_than_the_cores(multiply, route, m, n, k, ea, eb):
+    """Products near and below FP32's normal range: the largest and the mean error, in absolute
+    terms, are at most the core's, whose every multiply-add rounds to a multiple of 2^-149."""
+    rng = np.random.Generator(np.random.PCG64(k - ea))
+    A, B = ((rng.uniform(0.5, 1.0, s) * rng.choice([-1.0, 1.0], s) * 2.0**e).astype(np.float32)
+            for s, e in (((m, k), ea), ((k, n), eb)))
+    want = A.astype(np.float64) @ B.astype(np.float64)
+    err = {r: np.abs(multiply(r, A, B) - want) for r in ("core", route)}
+    assert err[route].max() <= err["core"].max()
+    assert err[route].mean() <= err["core"].mean()
