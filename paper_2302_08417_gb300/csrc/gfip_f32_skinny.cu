@@ -17,7 +17,7 @@
 //              slower; two groups of eight taking turns at the blocks, 35 %.)
 // Partial sums of all k ranges are added, in order, by a launch of its own, which also applies
 // alpha and beta: C is untouched when an element outside the range of the split turned up and
-// the FFMA launch behind has to compute the product.
+// the FFMA launch behind has to compute the product.  Every CTA then stops at its next look.
 //
 // Measured: 64 x 8192 x 8192 207 us from planes -> 120 to 129 here.
 // Bound: the latencies of the split (about 1550 clocks a block, for 600 of its instructions, 770
@@ -71,6 +71,9 @@ __device__ void producer(const SkinnyParams &p, tc::Smem &sm)
         const Unit x = unit_of(p, u);
         const uint8_t *src = p.planes + (int64_t)x.kb0 * PLANES * PLANE_BYTES;
         for (int kb = x.kb0; kb < x.kb1; ++kb, src += PLANES * PLANE_BYTES) {
+            // another CTA met an element outside the range: stop (no wait has run out)
+            if ((kb & 7) == 7 && leader && *(volatile const unsigned int *)p.gate != 0u)
+                tc::set_aborted(sm);
             ok = tc::mbar_wait(&sm.aempty[stage], (lap & 1u) ^ 1u, sm, p.status, p.wait_ns);
             if (!ok) break;
             if (leader && !skip) {
@@ -196,6 +199,12 @@ struct Block {
     }
 };
 
+// An element met so far lies outside the range of the split.
+__device__ __forceinline__ bool outside(uint32_t high, uint32_t low)
+{
+    return high >= tc::HIGH_BITS || low < tc::LOW_BITS - 1u;
+}
+
 // A wait that gives up has raised the abort flag, and every later one returns at once; the unit
 // is run to its end all the same (its result is invalid, its accesses are the same), so that the
 // lanes of a warp stay together for the warp-wide instructions, and the warp leaves after it.  (A
@@ -254,7 +263,19 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
             src += step;
             left -= KB;
         }
+        // blocks before the next look at what has been split so far: 3, 6, 12, 24, 48, 72 ...
+        int check = DEPTH;
+        bool stopped = false;
         for (int b0 = 0; b0 < len; b0 += DEPTH) {
+            if (b0 == check) {
+                check += min(check, 8 * DEPTH);
+                const bool stop = outside(high, low) || tc::aborted(sm);
+                stopped = __any_sync(0xffffffffu, stop) != 0;
+                if (stopped) {   // the product is the launch's behind: no more of it here
+                    tc::set_aborted(sm);
+                    break;
+                }
+            }
 #pragma unroll
             for (int d = 0; d < DEPTH; ++d) {
                 const int b = b0 + d;   // block within the unit
@@ -276,8 +297,8 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
                 left -= KB;
             }
         }
-        drain_to((len + p.chunk - 1) / p.chunk);
-        ok = __all_sync(0xffffffffu, ok) != 0;
+        if (!stopped) drain_to((len + p.chunk - 1) / p.chunk);
+        ok = __all_sync(0xffffffffu, ok && !stopped) != 0;
         if (!ok) break;
         // partial sums of the unit: [small row][128 rows of the large operand]
         float *out = p.partial + ((int64_t)u * p.n16 + part * cols) * TM + quarter * 32 + lane;
@@ -285,8 +306,7 @@ __device__ void splitter(const SkinnyParams &p, tc::Smem &sm, uint32_t tmem)
         for (int c = 0; c < 32; ++c)
             if (c < cols) __stcg(out + c * TM, acc[c]);
     }
-    const bool bad = high >= tc::HIGH_BITS || low < tc::LOW_BITS - 1u;
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(p.gate, 1u);
+    if (__any_sync(0xffffffffu, outside(high, low)) && lane == 0) atomicOr(p.gate, 1u);
 }
 
 __global__ void __launch_bounds__(THREADS, 1) skinny_kernel(const SkinnyParams p)
@@ -318,15 +338,19 @@ __global__ void __launch_bounds__(THREADS, 1) skinny_kernel(const SkinnyParams p
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc::tc_fence_before();
-    __syncthreads();
+    // an element of the small operand lies outside the range, or another CTA has met one
+    const bool skip =
+        __syncthreads_or(tid == 0 && *(volatile const unsigned int *)p.gate != 0u) != 0;
     tc::tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    if (warp == 0)
-        producer(p, sm);
-    else if (warp == 1)
-        issuer(p, sm, tmem);
-    else
-        splitter(p, sm, tmem);
+    if (!skip) {
+        if (warp == 0)
+            producer(p, sm);
+        else if (warp == 1)
+            issuer(p, sm, tmem);
+        else
+            splitter(p, sm, tmem);
+    }
     tc::tc_fence_before();
     __syncwarp();
     __syncthreads();

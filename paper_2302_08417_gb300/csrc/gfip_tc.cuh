@@ -87,6 +87,11 @@ __device__ __forceinline__ bool aborted(const Smem &sm)
     return *(volatile const int *)&sm.abort != 0;
 }
 
+__device__ __forceinline__ void set_aborted(Smem &sm)
+{
+    *(volatile int *)&sm.abort = 1;
+}
+
 __device__ __forceinline__ uint32_t saddr(const void *p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -143,7 +148,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Smem &
         if (aborted(sm)) return false;
         if ((it & 63) == 63 && global_ns() - t0 > budget_ns) break;
     }
-    *(volatile int *)&sm.abort = 1;
+    set_aborted(sm);
     atomicOr(status, sm.timeout_bit);
     return false;
 }

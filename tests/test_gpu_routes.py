@@ -163,3 +163,24 @@ def test_outside_the_planes_range_equals_the_core(routed, value):
     p = inputs.problem(7, "N", "N", 300, 280, 260, 1.0, 0.5, 7, 7, 7, dtype=F32)
     gu.assert_close(p, tensor.run(p)[0])
     assert core.h.status() == tensor.h.status() == skinny.h.status() == 0
+
+
+@pytest.mark.parametrize("at", [0, 700, 3499, "many", "small operand"])
+def test_few_rows_stop_at_an_element_outside(routed, at):
+    """The kernel for few rows stops where its CTAs next look (units of several looks, more units
+    than CTAs): the core's bits, C scaled once, no status, and the next call is right."""
+    core, skinny = routed("core"), routed("skinny")
+    for m, n, k in ((2000, 64, 3500), (25000, 16, 3500)):
+        p = inputs.problem(3, "N", "N", m, n, k, 1.0, 0.5, 0, 0, 0, dtype=F32)
+        clean_A, clean_B = p.A.copy(), p.B.copy()
+        if at == "small operand":
+            p.B[5] = 1e-42
+        elif at == "many":
+            p.A[::1001] = 1e-42
+        else:
+            p.A[m // 2 + at * m] = 1e-42
+        got, _ = skinny.run(p)
+        assert np.array_equal(got.view(np.uint8), core.run(p)[0].view(np.uint8))
+        p.A, p.B = clean_A, clean_B
+        gu.assert_close(p, skinny.run(p)[0])
+        assert skinny.h.status() == 0
