@@ -142,6 +142,11 @@ int gfip_set_pack_policy(gfip_handle_t handle, int policy);
  * GFIP_ERR_ARG for an unknown value.  The result bits do not depend on the packer. */
 int gfip_set_packer(gfip_handle_t handle, int packer);
 
+/* Large FP32 products on the tensor cores, from BF16 planes (see above): allowed (enable != 0, the
+ * default) or not.  When not, the FP32 kernel computes them, and the workspace-size queries leave
+ * the planes' room out: a workspace of that size serves the handle in either state. */
+int gfip_set_planes(gfip_handle_t handle, int enable);
+
 /* Fused-in-packing GEMM (the method of Sec. 3.2), FP64 and FP32. */
 int gfip_dgemm(gfip_handle_t handle, char transa, char transb, int64_t m, int64_t n, int64_t k,
                double alpha, const double *A, int64_t lda, const double *B, int64_t ldb,

@@ -50,6 +50,7 @@ struct Handle {
     size_t ctrl_bytes = 0;
     int pack_policy = GFIP_PACK_AUTO;
     int packer = GFIP_PACKER_AUTO;
+    bool planes = true;                            // gfip_set_planes
     unsigned long long oz_wait_ns = kOzakiWaitNs;  // budget of the emulation kernel's waits
     int oz_inject = 0;                             // test hook (gfip_debug_ozaki_timeout)
     unsigned long long f32_wait_ns = kF32WaitNs;   // budget of the FP32 kernels' waits
@@ -263,7 +264,7 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
                bool masked = false)
 {
     TcPlan t;
-    if (sizeof(T) != 4 || k > kTcMaxK || k < kTcMinK) return t;
+    if (sizeof(T) != 4 || !h->planes || k > kTcMaxK || k < kTcMinK) return t;
     t.use = h->route != GFIP_ROUTE_CORE;
     t.mt = static_cast<int>((m + 127) / 128);
     t.nt = static_cast<int>((n + 127) / 128);
@@ -1127,6 +1128,14 @@ int gfip_set_packer(gfip_handle_t handle, int packer)
     if (h == nullptr) return GFIP_ERR_HANDLE;
     if (packer < GFIP_PACKER_AUTO || packer > GFIP_PACKER_SHARED) return GFIP_ERR_ARG;
     h->packer = packer;
+    return GFIP_OK;
+}
+
+int gfip_set_planes(gfip_handle_t handle, int enable)
+{
+    Handle *h = get(handle);
+    if (h == nullptr) return GFIP_ERR_HANDLE;
+    h->planes = enable != 0;
     return GFIP_OK;
 }
 

@@ -56,6 +56,7 @@ SIGNATURES = {
     "gfip_set_workspace": (_int, [_ptr, _ptr, _sz]),
     "gfip_set_pack_policy": (_int, [_ptr, _int]),
     "gfip_set_packer": (_int, [_ptr, _int]),
+    "gfip_set_planes": (_int, [_ptr, _int]),
     "gfip_dgemm": (_int, _GEMM_D),
     "gfip_sgemm": (_int, _GEMM_S),
     "gfip_dgemm_direct": (_int, _GEMM_D),
@@ -166,6 +167,10 @@ def gfip_set_pack_policy(handle: int, policy: int) -> int:
 
 def gfip_set_packer(handle: int, packer: int) -> int:
     return load().gfip_set_packer(handle, packer)
+
+
+def gfip_set_planes(handle: int, enable: bool) -> int:
+    return load().gfip_set_planes(handle, int(bool(enable)))
 
 
 def _gemm_call(name, handle, transa, transb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc):
@@ -331,6 +336,7 @@ class Handle:
         self._device = torch.cuda.current_device
         self.h = gfip_create()
         self.workspace = None
+        self._short = None     # the smallest workspace there was no memory for
         self.stream = None
         if workspace_bytes:
             self._set_ws(workspace_bytes)
@@ -342,33 +348,59 @@ class Handle:
         if rc != GFIP_OK:
             raise GemmError(rc, "gfip_set_workspace")
 
+    def _grow(self, size, *args):
+        """A workspace for the calls that ``size`` (a workspace-size query) measures.  Where device
+        memory has no room for it, the smaller one that serves them without the split planes of
+        the FP32 tensor-core path (the FP32 kernel then computes them)."""
+        need = size(self.h, *args)
+        held = self.workspace
+        if held is not None:
+            if self._short is not None and need >= self._short and \
+                    held.numel() >= self._without_planes(size, *args):
+                return     # short of memory before, and this one does
+            self._torch.cuda.current_stream().synchronize()
+        try:
+            # room for somewhat larger calls, without doubling what a large one takes
+            self._set_ws(need + min(need // 4, 1 << 30) + (1 << 20))
+        except self._torch.cuda.OutOfMemoryError:
+            gfip_set_workspace(self.h, 0, 0)
+            held = self.workspace = None     # the next one may need its room
+            self._short = need if self._short is None else min(need, self._short)
+            self._set_ws_first_that_fits(need, self._without_planes(size, *args))
+
+    def _without_planes(self, size, *args):
+        gfip_set_planes(self.h, False)
+        need = size(self.h, *args)
+        gfip_set_planes(self.h, True)
+        return need
+
+    def _set_ws_first_that_fits(self, *sizes):
+        for n in sizes[:-1]:
+            try:
+                return self._set_ws(n)
+            except self._torch.cuda.OutOfMemoryError:
+                pass
+        self._set_ws(sizes[-1])
+
     def ensure_workspace(self, transa, transb, m, n, k, elem_bytes):
         need = gfip_workspace_size(self.h, transa, transb, m, n, k, elem_bytes)
         if self.workspace is None or self.workspace.numel() < need:
-            if self.workspace is not None:
-                self._torch.cuda.current_stream().synchronize()
-            self._set_ws(int(need * 1.25) + (1 << 20))
+            self._grow(gfip_workspace_size, transa, transb, m, n, k, elem_bytes)
 
     def ensure_syrk_workspace(self, uplo, trans, n, k, elem_bytes):
         need = gfip_syrk_workspace_size(self.h, uplo, trans, n, k, elem_bytes)
         if self.workspace is None or self.workspace.numel() < need:
-            if self.workspace is not None:
-                self._torch.cuda.current_stream().synchronize()
-            self._set_ws(int(need * 1.25) + (1 << 20))
+            self._grow(gfip_syrk_workspace_size, uplo, trans, n, k, elem_bytes)
 
     def ensure_trmm_workspace(self, side, uplo, transa, diag, m, n, elem_bytes):
         need = gfip_trmm_workspace_size(self.h, side, uplo, transa, diag, m, n, elem_bytes)
         if self.workspace is None or self.workspace.numel() < need:
-            if self.workspace is not None:
-                self._torch.cuda.current_stream().synchronize()
-            self._set_ws(int(need * 1.25) + (1 << 20))
+            self._grow(gfip_trmm_workspace_size, side, uplo, transa, diag, m, n, elem_bytes)
 
     def ensure_trsm_workspace(self, side, uplo, transa, diag, m, n, elem_bytes):
         need = gfip_trsm_workspace_size(self.h, side, uplo, transa, diag, m, n, elem_bytes)
         if self.workspace is None or self.workspace.numel() < need:
-            if self.workspace is not None:
-                self._torch.cuda.current_stream().synchronize()
-            self._set_ws(int(need * 1.25) + (1 << 20))
+            self._grow(gfip_trsm_workspace_size, side, uplo, transa, diag, m, n, elem_bytes)
 
     def bind_stream(self, stream=None):
         # the raw handle of torch's current stream: building the Stream object takes 2.8 us,
