@@ -323,21 +323,38 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
 
 // Whether a product runs on the small kernels (gfip_small.cu).
 //
-// FP64: everywhere but where the persistent core is as fast.  Above 2^35 multiply-adds both are
-// DFMA-bound within 0.1 % (4096^3: 109.9 and 110.0 ms) and the core draws a tenth of the L2
-// traffic; with few terms per element of a large C its 32 x 32 tiles cost less around the
-// arithmetic (8192 x 8192 x 64: 7.19 ms against 7.27; 1500 x 1500 x 64: 272 us against 251).
+// FP64: everywhere, but from k = 8192 on only where its estimated clocks are no more than the
+// persistent core's.  That core pads to 32 x 32 tiles and adds a tile's parts one after the other
+// (8 x 8 x 30000 takes it 807 us, the small kernel 83), but keeps all SMs busy on few tiles and a
+// long k: 8 x 8 x 4000000 7.6 ms against 16 to 23, 128 x 128 x 200000 5.4 against 5.5 to 6.0.
+// Above 2^35 multiply-adds both are DFMA-bound within 0.1 % (4096^3: 109.9 and 110.0 ms) and the
+// core draws a tenth of the L2 traffic; with few terms per element of a large C its tiles cost
+// less around the arithmetic (8192 x 8192 x 64: 7.19 ms against 7.27; 1500 x 1500 x 64: 272 us
+// against 251), and of a triangle, whose masked small kernel is slower, sooner (SYRK 4000 x 8:
+// 261 us against 388, 4000 x 64 908 against 1035; 1500 x 64 145 against 152, 1500 x 300 613
+// against 587).
 //
 // FP32: where the estimated time, in ns, is below the tensor cores' (or the FFMA core's, where
 // those cannot be used).  The estimates are fits on one GB300: 512^3 takes 14 us here and 17 on
 // the tensor cores, 640^3 24 and 18, 2000 x 2000 x 16 33 and 16 (23 on the FFMA core).
 template <typename T>
-bool use_small(const Handle *h, const TcPlan &tc, int64_t m, int64_t n, int64_t k, int tri)
+bool use_small(const Handle *h, const TcPlan &tc, char transa, char transb, int64_t m, int64_t n,
+               int64_t k, int tri)
 {
     if (h->route != GFIP_ROUTE_AUTO) return h->route == GFIP_ROUTE_SMALL;
     const double work = (double)m * n * k, part = tri ? 0.5 : 1.0;
-    if (sizeof(T) == 8)
-        return work <= (double)(1ll << 35) && (k > 64 || (double)m * n <= (double)(1 << 24));
+    if (sizeof(T) == 8) {
+        if (work > (double)(1ll << 35)) return false;
+        if (tri ? 8 * k <= m && m > 2048 : k <= 64 && (double)m * n > (double)(1 << 24))
+            return false;
+        if (k < 8192) return true;
+        const double mt = (double)((m + 31) / 32), nt = (double)((n + 31) / 32);
+        const double tiles = tri ? mt * (mt + 1) / 2 : mt * nt;
+        const double parts = std::floor(6.0 * h->sms / tiles);   // of one tile, if more than one
+        const double core = 1.045 * tiles * k * 1024 / (2 * h->sms) + 1780 * parts;
+        return (double)gfip::small_dgemm_clocks(m, n, k, tri, is_notrans(transa) ? 1 : 0,
+                                                is_notrans(transb) ? 0 : 1, h->sms) <= core;
+    }
     const double tiles = part * (double)((m + 31) / 32) * ((n + 31) / 32);
     double small = std::numeric_limits<double>::max();
     for (int cs = 1; cs <= 8 && (cs == 1 || cs * 64 <= k); cs *= 2)
@@ -512,7 +529,7 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
     // A workspace too small for the split planes still serves the FFMA path.
     TcPlan tc = tc_plan<T>(h, transa, transb, m, n, k, tri, tmask_a || tmask_b);
     tc.use = tc.use && call_bytes(h, pl, tc) <= ws_limit;
-    if (use_small<T>(h, tc, m, n, k, tri)) {
+    if (use_small<T>(h, tc, transa, transb, m, n, k, tri)) {
         const gfip::SmallParams<T> sp{A, B, C, lda, ldb, ldc, (int)m, (int)n, (int)k, alpha, beta,
                                       is_notrans(transa) ? 1 : 0, is_notrans(transb) ? 0 : 1,
                                       tri, tmask_a, tmask_b, 0, 0};

@@ -266,6 +266,9 @@ template <typename T> struct SmallParams {
     int mt, tiles;                // tiles along m, and of C (set by the launcher)
 };
 template <typename T> cudaError_t launch_small(SmallParams<T> p, int sms, cudaStream_t s, int *grid);
+// Estimated clocks of the FP64 kernel.
+int64_t small_dgemm_clocks(int64_t m, int64_t n, int64_t k, int tri, int a_contig_m,
+                           int b_contig_n, int sms);
 
 // Launchers (defined per element type in gfip_f64.cu / gfip_f32.cu).
 template <typename T> cudaError_t launch_gemm(const GemmParams<T> &p, cudaStream_t s);

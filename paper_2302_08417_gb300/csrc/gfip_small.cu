@@ -385,23 +385,55 @@ __global__ void __launch_bounds__(SWARPS * 32, 2) sgemm_kernel(const SmallParams
     }
 }
 
-// CTAs per tile: the fewest clocks on the busiest SM, where a CTA takes `per_k` clocks per k and
-// about `fixed` around its k loop, a cluster 1500 more.
+// Clocks on the busiest SM with cs CTAs per tile: a CTA takes `per_k` clocks per k and about `fixed`
+// around its k loop, a cluster 1500 more.  `wait`: clocks per k that its loads take beyond that.
+inline int64_t clocks_of(int cs, int64_t tiles, int64_t k, int64_t per_k, int64_t fixed,
+                         int64_t wait, int sms)
+{
+    const int64_t rounds = (tiles * cs + sms - 1) / sms;
+    // the other CTAs of the SM hide the wait
+    return (k + cs - 1) / cs * std::max(rounds * per_k, per_k + wait) + rounds * fixed +
+           (cs > 1 ? 1500 : 0);
+}
+
+// CTAs per tile: the fewest clocks.
 inline int cluster_size(int64_t tiles, int64_t k, int64_t group, int64_t per_k, int64_t fixed,
-                        int sms)
+                        int64_t wait, int sms)
 {
     int best = 1;
     int64_t least = 0;
     for (int cs = 1; cs <= 8; cs *= 2) {
         if (cs > 1 && cs * group > k) break;
-        const int64_t rounds = (tiles * cs + sms - 1) / sms;
-        const int64_t cost = rounds * ((k + cs - 1) / cs * per_k + fixed) + (cs > 1 ? 1500 : 0);
+        const int64_t cost = clocks_of(cs, tiles, k, per_k, fixed, wait, sms);
         if (cs == 1 || cost < least) {
             best = cs;
             least = cost;
         }
     }
     return best;
+}
+
+// FP64: a CTA's 8 x 8 tile takes 32 DFMA clocks per k.
+constexpr int64_t DCLOCKS = 32, DFIXED = 1000;
+
+// Its warps load one group ahead.  Alone on its SM a CTA waits 10 clocks per k more for L2
+// (8 x 8 x 200000: 313 ns a step), and up to 36 for HBM, where operands come from that do not stay
+// in L2 (from about 50 to 60 MB on), or 60 when one lies along k and the other across (8 x 8 x
+// 4000000: 560 and 730 ns a step).
+inline int64_t dgemm_wait(int64_t mb, bool mixed)
+{
+    return mixed ? std::min<int64_t>(60, 14 + std::max<int64_t>(0, mb - 50) * 7 / 4)
+                 : std::min<int64_t>(36, 10 + std::max<int64_t>(0, mb - 64) * 2 / 3);
+}
+
+// CTAs per tile, FP64: by the DFMA clocks, and by the wait as well where it is HBM's.  (By the DFMA
+// clocks alone, 64 x 64 x 200000 ran on 128 CTAs in 3.1 to 4.0 ms.)
+inline int dgemm_cluster(int64_t run, int64_t m, int64_t n, int64_t k, int tri, bool mixed,
+                         int sms)
+{
+    const int64_t mb = ((tri == TRI_NONE ? m + n : m) * k) >> 17;
+    return cluster_size(run, k, DWARPS * U, DCLOCKS, DFIXED, mb > 50 ? dgemm_wait(mb, mixed) : 0,
+                        sms);
 }
 
 // Tiles that are not left out: about half of a triangle's square.
@@ -472,6 +504,24 @@ cudaError_t launch_any(const SmallParams<T> &p, unsigned int blocks, int cs, cud
 
 }  // namespace small
 
+int64_t small_dgemm_clocks(int64_t m, int64_t n, int64_t k, int tri, int a_contig_m,
+                           int b_contig_n, int sms)
+{
+    using namespace small;
+    const int64_t run = computed((m + DT - 1) / DT * ((n + DT - 1) / DT), tri);
+    const bool mixed = a_contig_m != b_contig_n;
+    const int cs = dgemm_cluster(run, m, n, k, tri, mixed, sms);
+    const int64_t mb = ((tri == TRI_NONE ? m + n : m) * k) >> 17;
+    const int64_t wait = dgemm_wait(mb, mixed), rounds = (run * cs + sms - 1) / sms;
+    const int64_t clocks = clocks_of(cs, run, k, DCLOCKS, DFIXED, wait, sms);
+    // large clusters over HBM do not spread evenly (128 x 64 x 500000: 7900 us, 6750 by the rounds)
+    if (tri == TRI_NONE) return cs >= 4 && rounds > 2 && mb > 128 ? clocks + clocks / 6 : clocks;
+    // the masked kernel's loads wait longer, most where both operands lie across k (SYRK 16 x
+    // 300000 993 us along, 1512 across), and its CTAs hide little of it (64 x 64 x 300000 2343)
+    return (k + cs - 1) / cs * (rounds * DCLOCKS + wait + (a_contig_m ? 40 : 15)) +
+           rounds * DFIXED;
+}
+
 template <> cudaError_t launch_small<double>(SmallParams<double> p, int sms, cudaStream_t s,
                                                int *grid)
 {
@@ -480,15 +530,19 @@ template <> cudaError_t launch_small<double>(SmallParams<double> p, int sms, cud
     const int64_t tiles = (int64_t)p.mt * ((p.n + DT - 1) / DT);
     p.tiles = static_cast<int>(tiles);
     const int64_t run = computed(tiles, p.tri);
-    int cs = cluster_size(run, p.k, DWARPS * U, 32, 1000, sms);
+    const bool mixed = p.a_contig_m != p.b_contig_n, across = p.a_contig_m && p.b_contig_n;
+    int cs = dgemm_cluster(run, p.m, p.n, p.k, p.tri, mixed, sms);
     // A tile per warp, where there are enough, all are whole and no DFMA clocks are lost on the
     // busiest unit: 64 a row of k and element; 10 instructions end a shared tile (on one unit,
     // while the others go on), 4 an own one.  Within 1 % the own tile is taken, whose sums are
-    // one chain in k order like the persistent core's.
+    // one chain in k order like the persistent core's; but not for a long k across which both
+    // operands lie, where a warp's loads of a step touch 32 lines for its tile alone (N/T, us:
+    // 500 x 1000 x 10000 9327 own, 8132 shared, 8586 the core; 1000^3 1688 and 1625; but
+    // 4000 x 4000 x 100 2671 and 2833).
     const int64_t shared = (run + sms - 1) / sms * (p.k * 32 + 160);
     const int64_t own = (run + 4 * sms - 1) / (4 * sms) * (p.k * 128 + 256);
     const bool masked = p.tri != TRI_NONE || p.tmask_a || p.tmask_b;
-    if (cs == 1 && !masked && run >= 16 * sms && own * 100 <= shared * 101)
+    if (cs == 1 && !masked && !(across && p.k >= 512) && run >= 16 * sms && own * 100 <= shared * 101)
         cs = 0;
     const int64_t blocks = cs == 0 ? (tiles + DWARPS - 1) / DWARPS : tiles;
     *grid = static_cast<int>(blocks * std::max(cs, 1));
@@ -500,7 +554,7 @@ template <> cudaError_t launch_small<float>(SmallParams<float> p, int sms, cudaS
     using namespace small;
     p.mt = (p.m + ST - 1) / ST;
     const int64_t tiles = (int64_t)p.mt * ((p.n + ST - 1) / ST);
-    const int cs = cluster_size(computed(tiles, p.tri), p.k, SK, 22, 1500, sms);
+    const int cs = cluster_size(computed(tiles, p.tri), p.k, SK, 22, 1500, 0, sms);
     *grid = static_cast<int>(tiles * cs);
     return launch_any(p, static_cast<unsigned int>(tiles), cs, s);
 }
