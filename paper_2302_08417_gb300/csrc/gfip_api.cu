@@ -247,11 +247,29 @@ template <typename T> size_t total_bytes(Handle *h, const Plan<T> &pl)
     return ctrl + pl.data_bytes;
 }
 
+// k blocks (of 32) per accumulation of an FP32 product on the tensor cores, whose FFMA plan is pl.
+//
+// The tensor cores' truncation shows as a bias that grows with a chunk's length, the FFMA core's
+// error grows with its chains' length L and shrinks as more of them are added; the chunks are so
+// short that the first is the smaller.  Entries in [0, 1], relative error in 1e-8: chunks of 32 k 5
+// to 6, 64 k 8, 128 k 14.5 (the sum of many chunks adds to it: 12 for 64 k at k = 2500); the FFMA
+// core about sqrt(2 L^2 / k + 30): one chain of 128 16, of 1024 30; 512 x 512 x 1500 in twelve
+// chains of 128 7.3, 1030 x 1100 x 1500 in four of 400 14.7.  Short chunks cost drains: 4096^3 takes
+// 710 us with 64, 651 with 128; 512 x 512 x 4096 43 with 32 and 41 with 64.
+int tc_chunk(const Plan<float> &pl, int64_t k)
+{
+    const double chain =
+        pl.dp_tiles > 0 ? (double)k : std::min<double>(k, 32.0 * pl.sk_iters / pl.grid);
+    const double spread = chain * chain / k;
+    return k > 1024 && spread >= 128 ? 4 : k > 512 && spread < 22 ? 1 : 2;
+}
+
 // A large FP32 product on the tensor cores (gfip_f32_tc.cu): the split pass, then the tile
 // core over the plane tiles, k split over `splits` units per tile.
 struct TcPlan {
     bool use = false;
     int mt = 0, nt = 0, kt = 0, tiles = 0, splits = 1;
+    int chunk = 1;      // k blocks per accumulation
     int64_t cost = 0;   // k blocks in a row on the busiest SM, overheads counted as blocks
     double ns = 0;      // estimated time
     size_t off_a = 0, off_b = 0, off_partial = 0, off_counter = 0, data_bytes = 0;
@@ -260,8 +278,8 @@ struct TcPlan {
 };
 
 template <typename T>
-TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, int64_t k, int tri,
-               bool masked = false)
+TcPlan tc_plan(const Handle *h, const Plan<T> &pl, char transa, char transb, int64_t m, int64_t n,
+               int64_t k, int tri, bool masked = false)
 {
     TcPlan t;
     if (sizeof(T) != 4 || !h->planes || k > kTcMaxK || k < kTcMinK) return t;
@@ -270,6 +288,7 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
     t.nt = static_cast<int>((n + 127) / 128);
     t.kt = static_cast<int>((k + 31) / 32);
     t.tiles = tri ? t.mt * (t.mt + 1) / 2 : t.mt * t.nt;
+    if constexpr (sizeof(T) == 4) t.chunk = tc_chunk(pl, k);
     // The units of one tile run on different SMs.  Fewest k blocks in a row on the busiest SM,
     // each unit costing about 6 more (pipeline fill, epilogue), a split tile 2 per part added.
     t.cost = std::numeric_limits<int64_t>::max();
@@ -281,20 +300,24 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
             t.splits = s;
         }
     }
-    // Estimated times, ns, fitted to one GB300: 640^3 19 us, 2048^3 106, 300 x 290 x 2500 31 (28 on
-    // the small kernel), 64 x 8192 x 8192 212 (its planes' 10 bytes an element dominate) and, split
-    // on the way, 120; 100 x 2000 x 2000 32 and 39.
-    const double planes = (double)m * k + (tri ? 0.0 : (double)n * k);
+    // Estimated times, ns, fitted to one GB300 (us, measured): 640^3 19, 2048^3 106,
+    // 300 x 290 x 2500 31, 8 x 8 x 60000 138, 128 x 500 x 30000 104 (planes of whole 128-row blocks
+    // at 10 bytes an element, and where chunks are one block their drains), 64 x 8192 x 8192 212
+    // and, split on the way, 120; 100 x 2000 x 2000 32 and 39, 128 x 500 x 30000 118, 8 x 8 x 60000
+    // 118.
+    const double planes = 128.0 * (t.mt + (tri ? 0 : t.nt)) * k;
     const double part = tri ? 0.5 : 1.0;
     const int64_t in_a_row = ((int64_t)t.tiles * t.splits + h->sms - 1) / h->sms *
                              ((t.kt + t.splits - 1) / t.splits);
-    t.ns = 9000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost + 130.0 * in_a_row;
+    t.ns = 9000 + 0.002 * planes + 0.0016 * part * m * n + 400.0 * t.cost +
+           (t.chunk == 1 ? 300.0 : 130.0) * in_a_row;
     // at most 128 rows or columns against an operand that is read along memory: k blocks on the
     // busiest SM, and the launch that adds the k ranges
     if (tri == gfip::TRI_NONE && !masked && std::min(m, n) <= 128 &&
         (n <= m ? is_notrans(transa) : !is_notrans(transb))) {
         const int n16 = static_cast<int>((std::min(m, n) + 15) / 16 * 16);
-        const double ns = 17000 + (double)in_a_row * (600 + 3.2 * n16) + 1000.0 * t.splits;
+        const double ns = 17000 + (double)in_a_row * (600 + (t.chunk == 1 ? 6.0 : 3.2) * n16) +
+                          1000.0 * t.splits;
         if (h->route == GFIP_ROUTE_SKINNY || (ns < t.ns && h->route != GFIP_ROUTE_TENSOR)) {
             t.skinny = true;
             t.n16 = n16;
@@ -335,8 +358,10 @@ TcPlan tc_plan(const Handle *h, char transa, char transb, int64_t m, int64_t n, 
 // against 587).
 //
 // FP32: where the estimated time, in ns, is below the tensor cores' (or the FFMA core's, where
-// those cannot be used).  The estimates are fits on one GB300: 512^3 takes 14 us here and 17 on
-// the tensor cores, 640^3 24 and 18, 2000 x 2000 x 16 33 and 16 (23 on the FFMA core).
+// those cannot be used).  The estimates are fits on one GB300: 512^3 takes 14 us here and 20 on
+// the tensor cores, 640^3 25 and 19, 2000 x 2000 x 16 39 and 12 (19 on the FFMA core); a slab of 64
+// k takes 750 ns, more when clusters wait for it (8 x 8 x 30000 870, 128 x 128 x 30000 1390,
+// 128 x 500 x 30000, from HBM, 950 to 1200).
 template <typename T>
 bool use_small(const Handle *h, const TcPlan &tc, char transa, char transb, int64_t m, int64_t n,
                int64_t k, int tri)
@@ -357,10 +382,14 @@ bool use_small(const Handle *h, const TcPlan &tc, char transa, char transb, int6
     }
     const double tiles = part * (double)((m + 31) / 32) * ((n + 31) / 32);
     double small = std::numeric_limits<double>::max();
-    for (int cs = 1; cs <= 8 && (cs == 1 || cs * 64 <= k); cs *= 2)
-        small = std::min(small, 2500 + std::ceil(tiles * cs / h->sms) *
-                                           (400 + 750 * std::ceil((double)k / (64 * cs))) +
+    for (int cs = 1; cs <= 8 && (cs == 1 || cs * 64 <= k); cs *= 2) {
+        const double rounds = std::ceil(tiles * cs / h->sms);
+        const double slab = cs == 1       ? 750
+                            : rounds == 1 ? 750 + 5 * tiles * cs
+                                          : (m + n) * k > (15 << 20) ? 1150 : 750;
+        small = std::min(small, 2500 + rounds * (400 + slab * std::ceil((double)k / (64 * cs))) +
                                     (cs > 1 ? 800 : 0));
+    }
     if (!tc.use) return small < 12000 + 0.00265 * part * m * n + 8e-5 * part * work;
     return small < tc.ns;
 }
@@ -434,18 +463,6 @@ int gemm_entry(gfip_handle_t handle, Variant v, char transa, char transb, int64_
 cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<float> &p,
                       unsigned char *data)
 {
-    // k blocks (of 32) per accumulation on the tensor cores, whose truncation shows as a bias that
-    // grows with a chunk's length, to be no further off than the FFMA core, whose error grows with
-    // its chains' length L and shrinks as more of them are added.  Entries in [0, 1], relative
-    // error in 1e-8: chunks of 32 k 5 to 6, 64 k 8, 128 k 14.5 (with many chunks their sum adds
-    // to it: 12 for 64 k at k = 2500); the FFMA core about sqrt(2 L^2 / k + 30): one chain of 128
-    // 16, of 1024 30; 512 x 512 x 1500 in twelve chains of 128 7.3, 1030 x 1100 x 1500 in four of
-    // 400 14.7.  Short chunks cost drains: 4096^3 takes 710 us with 64, 651 with 128;
-    // 512 x 512 x 4096 43 with 32 and 41 with 64.
-    const double chain =
-        p.dp_tiles > 0 ? (double)p.k : std::min<double>(p.k, 32.0 * p.sk_iters / p.grid);
-    const double spread = chain * chain / p.k;
-    const int chunk = p.k > 1024 && spread >= 128 ? 4 : p.k > 512 && spread < 22 ? 1 : 2;
     if (t.skinny) {
         const bool big_is_row = p.n <= p.m;   // op(A) is the large operand
         gfip::SkinnyParams q{};
@@ -459,7 +476,7 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
         q.tiles = t.tiles;
         q.splits = t.splits;
         q.units = t.tiles * t.splits;
-        q.chunk = chunk;
+        q.chunk = t.chunk;
         q.partial = reinterpret_cast<float *>(data + t.off_partial);
         q.gate = p.gate;
         q.status = p.status;
@@ -495,7 +512,7 @@ cudaError_t launch_tc(const Handle *h, const TcPlan &t, const gfip::GemmParams<f
     q.tmask_b = p.tmask_b;
     q.splits = t.splits;
     q.units = t.tiles * t.splits;
-    q.chunk = chunk;
+    q.chunk = t.chunk;
     q.partial = reinterpret_cast<float *>(data + t.off_partial);
     q.counter = reinterpret_cast<unsigned int *>(data + t.off_counter);
     q.gate = p.gate;
@@ -527,7 +544,7 @@ int launch_plan(Handle *h, Variant v, int tri, char transa, char transb, int64_t
         return rc;
 
     // A workspace too small for the split planes still serves the FFMA path.
-    TcPlan tc = tc_plan<T>(h, transa, transb, m, n, k, tri, tmask_a || tmask_b);
+    TcPlan tc = tc_plan<T>(h, pl, transa, transb, m, n, k, tri, tmask_a || tmask_b);
     tc.use = tc.use && call_bytes(h, pl, tc) <= ws_limit;
     if (use_small<T>(h, tc, transa, transb, m, n, k, tri)) {
         const gfip::SmallParams<T> sp{A, B, C, lda, ldb, ldc, (int)m, (int)n, (int)k, alpha, beta,
@@ -705,7 +722,7 @@ size_t workspace_size_impl(Handle *h, char transa, char transb, int64_t m, int64
     if (too_big(m) || too_big(n) || too_big(k)) return 0;
     if (m == 0 || n == 0 || k == 0) return round_up(kHeader, kCtrlGranule);
     const Plan<T> pl = make_plan<T>(h, v, (int)m, (int)n, (int)k);
-    return call_bytes(h, pl, tc_plan<T>(h, transa, transb, m, n, k, gfip::TRI_NONE));
+    return call_bytes(h, pl, tc_plan<T>(h, pl, transa, transb, m, n, k, gfip::TRI_NONE));
 }
 
 // Reference-BLAS dsyrk argument check: 0, or minus the 1-based position of the first bad
@@ -769,7 +786,7 @@ size_t syrk_workspace_impl(Handle *h, char uplo, char trans, int64_t n, int64_t 
     if (n == 0 || k == 0) return round_up(kHeader, kCtrlGranule);
     const int tri = (uplo == 'L' || uplo == 'l') ? gfip::TRI_LOWER : gfip::TRI_UPPER;
     const Plan<T> pl = make_plan<T>(h, Variant::Fused, (int)n, (int)n, (int)k, tri);
-    return call_bytes(h, pl, tc_plan<T>(h, 'N', 'T', n, n, k, tri));
+    return call_bytes(h, pl, tc_plan<T>(h, pl, 'N', 'T', n, n, k, tri));
 }
 
 // Reference-BLAS dtrmm argument check: 0, or minus the 1-based position of the first bad
@@ -810,7 +827,7 @@ size_t trmm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
     const bool left = side == 'L' || side == 'l';
     const Plan<T> pl =
         make_plan<T>(h, Variant::Fused, (int)m, (int)n, (int)(left ? m : n), gfip::TRI_NONE, true);
-    const TcPlan tc = tc_plan<T>(h, 'N', 'N', m, n, left ? m : n, gfip::TRI_NONE, true);
+    const TcPlan tc = tc_plan<T>(h, pl, 'N', 'N', m, n, left ? m : n, gfip::TRI_NONE, true);
     return round_up(call_bytes(h, pl, tc), kAlign) + round_up((size_t)m * n * sizeof(T), kAlign);
 }
 
@@ -848,7 +865,8 @@ int trmm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     const size_t w_bytes = (size_t)m * n * sizeof(T);
     // a workspace without room for the split planes of the tensor-core path runs without it
     size_t w_off =
-        round_up(call_bytes(h, pl, tc_plan<T>(h, 'N', 'N', m, n, kdim, gfip::TRI_NONE, true)), kAlign);
+        round_up(call_bytes(h, pl, tc_plan<T>(h, pl, 'N', 'N', m, n, kdim, gfip::TRI_NONE, true)),
+                 kAlign);
     if (w_off + w_bytes > h->ws_bytes) w_off = round_up(total_bytes(h, pl), kAlign);
     if (w_off + w_bytes > h->ws_bytes) return GFIP_ERR_WORKSPACE;
     T *W = reinterpret_cast<T *>(h->ws + w_off);
@@ -919,7 +937,7 @@ size_t trsm_workspace_impl(Handle *h, char side, int64_t m, int64_t n)
             const int64_t um = left ? rest : m, un = left ? n : rest;
             const Plan<T> pl = make_plan<T>(h, Variant::Fused, (int)um, (int)un, (int)width);
             for (const char t : {'N', 'T'})
-                bytes = std::max(bytes, call_bytes(h, pl, tc_plan<T>(h, t, t, um, un, width,
+                bytes = std::max(bytes, call_bytes(h, pl, tc_plan<T>(h, pl, t, t, um, un, width,
                                                                      gfip::TRI_NONE)));
         };
         // forward, the unknowns after each whole panel; backward, those before each panel
