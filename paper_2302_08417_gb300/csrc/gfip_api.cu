@@ -983,14 +983,13 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
     const bool unit = diag == 'U' || diag == 'u';
     const int na = (int)(left ? m : n);
     const char ta = trans ? 'T' : 'N';
-    unsigned char *image = nullptr;   // FP32: where a panel's triangle is packed
+    size_t ctrl = 0;
     if (alpha != T(0)) {
         // The control words are cleared before the first launch, for all panels.  While the
         // stream is capturing they cannot be; a single packed panel, which needs no control
         // word, is then solved without them: its triangle lies behind the region a first call
         // would clear, and it reports no status, so it is staged without waits.
-        const size_t ctrl = trsm_ctrl<T>(h, side, lower_t, m, n);
-        image = h->ws + std::max(h->ctrl_bytes, ctrl);
+        ctrl = trsm_ctrl<T>(h, side, lower_t, m, n);
         if (const int rc = grow_ctrl(h, ctrl);
             rc != GFIP_OK && !(rc == GFIP_ERR_CAPTURE && na <= gfip::TRSM_PANEL))
             return rc;
@@ -1026,7 +1025,9 @@ int trsm_entry(gfip_handle_t handle, char side, char uplo, char transa, char dia
         const int nvec = (int)(left ? n : m);
         cudaError_t e;
         if constexpr (sizeof(T) == 4) {
-            // the packed triangle takes the bytes the update's GEMM uses afterwards
+            // the packed triangle lies behind the control words, in the bytes the update's GEMM
+            // uses afterwards
+            unsigned char *image = h->ws + std::max(h->ctrl_bytes, ctrl);
             e = gfip::launch_trsm_panel_f32(
                 Bp, vstride, estride, nvec, A, lda, trans, p0, pw, lower_t, left ? 0 : 1, unit,
                 reinterpret_cast<float *>(image),
