@@ -40,7 +40,7 @@ FFMA_FLOP_PER_CLK_PER_SM = 256    # 128 FFMA lanes per clock per SM
 SM_MAX_MHZ = 2070.0
 FP64_PEAK_GFLOPS = SMS * DFMA_FLOP_PER_CLK_PER_SM * SM_MAX_MHZ / 1e3   # 1258.6
 FP32_PEAK_GFLOPS = SMS * FFMA_FLOP_PER_CLK_PER_SM * SM_MAX_MHZ / 1e3   # 80547.8
-HBM_GBS = 6785.2
+HBM_GBS = 6703.8
 BF16_TFLOPS = 1945.7   # measured, cuBLAS 8192^3, burst
 F32_TENSOR_PEAK_GFLOPS = BF16_TFLOPS * 1e3 / 8   # FP32 from eight products of BF16 planes
 def workload(dtype="f64", size=8192, variant="fused") -> str:
@@ -53,7 +53,7 @@ WORKLOAD = workload()
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the FP64 GEMM
 # kernel on this workload, from a one-pass ncu capture of the full-size launch (summary in
 # profiles/); valid only while the kernel sources hash to kernel_hash.
-TRAFFIC = {"bytes_per_launch": 23.14e9 + 1.65e9, "kernel_hash": "26b705248ccb94c3"}
+TRAFFIC = {"bytes_per_launch": 23.21e9 + 1.65e9, "kernel_hash": "655c5fe6500512eb"}
 KERNEL_SOURCES = ["paper_2302_08417_gb300/csrc/gfip_kernels.cuh",
                   "paper_2302_08417_gb300/csrc/gfip_internal.h"]
 

@@ -6,7 +6,7 @@
 // a3 b1 + a2 b3 + a3 b2); the one product left out, a3 b3, is at most 2^-32 of |a b|, a 256th of
 // half an ulp, so a sum that one product dominates comes out rounded as a multiply-add rounds it.
 // (Without a2 b3 + a3 b2, up to 2^-24 of |a b|, 4 % of such sums were an ulp off and the worst
-// error was 1.5 times a multiply-add's; the two products cost 4096^3 20 %.)  a1 b1 and the
+// error was 1.7 times a multiply-add's; the two products cost 4096^3 20 %.)  a1 b1 and the
 // smaller products are accumulated apart, for 32 to 128 k at a time (launch_tc in gfip_api.cu),
 // and the chunks are added in FP32 with rounding to nearest, which keeps the sum at least as
 // exact as the FFMA core's chains of FP32 multiply-adds, also where all terms have one sign.

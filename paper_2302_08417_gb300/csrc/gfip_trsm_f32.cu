@@ -22,7 +22,7 @@
 // Bound: the chain, about 2000 clocks a block (500 to update the next block's rows, 1350 to
 // solve them), with the updates further down just behind it.  512 unknowns, 512 right-hand
 // sides: 67 -> 36 us with the packing launch; 2048 x 2048 with its updates 386 -> 266 us (with
-// the caller's copy of B; 277 since the updates' accumulations are shorter).
+// the caller's copy of B; 286 since the updates form more products in shorter accumulations).
 #include <cstdint>
 
 #include "gfip_internal.h"
