@@ -107,6 +107,45 @@ def test_trmm(routed, route, dtype):
     trmm.test_integer_bit_exact(runner, dtype)
 
 
+@pytest.mark.parametrize("route,dtype", [("core", F64), ("core", F32), ("tensor", F32)],
+                         ids=["core-f64", "core-f32", "tensor-f32"])
+def test_triangles_over_several_rounds(routed, route, dtype):
+    """More tiles than SMs, ragged: the tensor cores' triangular operands take their longest tiles
+    first and every other round backwards, the core packs panels that later rounds read."""
+    runner = routed(route)
+    rng = np.random.Generator(np.random.PCG64(31))
+    u = inputs.unit_roundoff(dtype)
+
+    def close(got, X, Y, C, alpha, beta, part=slice(None)):
+        # numpy's FP64 products and the result are each within (k + 2) u of the exact one
+        want = alpha * (X @ Y) + beta * C
+        bound = abs(alpha) * (np.abs(X) @ np.abs(Y)) + abs(beta) * np.abs(C)
+        assert np.all(np.abs(got - want)[part] <= (2 * (X.shape[1] + 2) * u * bound)[part])
+
+    for side, uplo, ta, diag in trmm.COMBOS:
+        m, n = (1650, 1910) if side == "L" else (1910, 1650)
+        A = trmm.poisoned(rng, 1650, 1653, uplo, diag, dtype)
+        B0 = inputs.colmajor(rng, m, n, m + 1, dtype)
+        got, guard = trmm.run(runner, side, uplo, ta, diag, m, n, 1.25, A, 1653, B0, m + 1)
+        assert np.all(np.isnan(guard))
+        D = trmm.dense_op(A.astype(np.float64), 1653, 1650, uplo, ta, diag)
+        B = inputs.as_matrix(B0.astype(np.float64), m, n, m + 1)
+        close(inputs.as_matrix(got.astype(np.float64), m, n, m + 1),
+              *((D, B) if side == "L" else (B, D)), np.zeros((m, n)), 1.25, 0.0)
+    for uplo, trans in itertools.product("LU", "NT"):
+        n, k = 2500, 333
+        A, lda, C0, ldc = syrk.make(17, uplo, trans, n, k, 7, dtype)
+        got, guard = syrk.run(runner, uplo, trans, n, k, 0.75, A, lda, 0.5, C0, ldc)
+        assert np.all(np.isnan(guard))
+        X = inputs.as_matrix(A.astype(np.float64), *((n, k) if trans == "N" else (k, n)), lda)
+        X = X if trans == "N" else X.T
+        C = inputs.as_matrix(C0.astype(np.float64), n, n, ldc)
+        G = inputs.as_matrix(got.astype(np.float64), n, n, ldc)
+        tri = np.tri(n, dtype=bool) if uplo == "L" else np.tri(n, dtype=bool).T
+        close(np.where(tri, G, 0), X, X.T, np.where(tri, C, 0), 0.75, 0.5, tri)
+        assert np.array_equal(G[~tri], C[~tri], equal_nan=True)   # the other triangle
+
+
 @pytest.mark.parametrize("route,dtype", MASKED, ids=ids(MASKED))
 def test_trsm(routed, route, dtype):
     runner = routed(route)
